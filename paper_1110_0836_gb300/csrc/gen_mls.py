@@ -309,6 +309,18 @@ def gen():
     w("  return r >= c ? t[r * (r + 1) / 2 + c] : t[c * (c + 1) / 2 + r];")
     w("}")
     w("")
+    w("// The product mls_accum_moments forms moment a from: wq[b] (b = 0: the weight")
+    w("// alone) times qg[g].")
+    w("__device__ __forceinline__ void mls_moment_split(int a, int& b, int& g) {")
+    w("  constexpr unsigned char t[kNM][2] = {")
+    sp = [split(alpha) for alpha in MOMENTS]
+    for k in range(0, len(sp), 10):
+        w("    " + ", ".join(f"{{{b + 1}, {g}}}" for b, g in sp[k:k + 10]) + ",")
+    w("  };")
+    w("  b = t[a][0];")
+    w("  g = t[a][1];")
+    w("}")
+    w("")
     # Cholesky
     w("// In-place Cholesky of the packed normal matrix.  On return the packed")
     w("// array holds L (strict lower part; the diagonal entries keep M_kk) and")

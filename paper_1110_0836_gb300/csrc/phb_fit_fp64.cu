@@ -2,15 +2,33 @@
 // double-precision GPU form.  It serves every particle when the precision is
 // PHB_FP64, and the particles that the FP32-mixed kernel routed to FP64.
 //
-// One thread per particle.  The 80 moments and 8 x 19 right-hand sides are
-// accumulated in a thread-private shared-memory region (FP64 registers would
-// not hold them), the normal matrix is assembled and factorised in place by
-// the same unrolled Cholesky as the mixed kernel, and only the linear and
-// quadratic coefficients are back-substituted.  Fits whose Jacobi-scaled
-// conditioning estimate exceeds 1e4 take one corrected semi-normal-equations
-// step (Bjorck): residuals r_j = (U_j - U_i) - p(q_j).c are recomputed from the
-// data, A^T W r is accumulated again and solved with the same factor, so the
-// error follows cond(A) rather than cond(A^T W A) = cond(A)^2.
+// What bounds it: GB300's FP64 pipe.  A warp's FP64 instruction takes 17-20 SM
+// cycles when all four sub-partitions issue them (measured: 34 with two busy,
+// 68 with one), about 80 times an FP32 one, so the kernel counts FP64
+// instructions and keeps four warps per SM at them; shared-memory traffic,
+// integer work and FP32 work disappear behind them.  A lattice fit (52
+// neighbours) is 267 FP64 instructions per neighbour (80 moments, 7 x 19
+// right-hand sides, 54 for offsets, weight and monomials) and ~3,900 for the
+// factorisation and the solves: 18,500, or 8.3-9.5 ms for 262,144 particles.
+// Comparisons, the test for a periodic wrap and the conditioning estimate run
+// on the integer and FP32 pipes for that reason.  Measured: 11.5 ms (FP64 pipe
+// 66% busy); with all sums in shared memory and two warps per SM it was 23.0 ms
+// (35%).
+//
+// Two ways to fit a particle, bit-identical (each sum and each substitution
+// takes its terms in the same order):
+//   * thread per particle (fit_thread): the 80 moments in registers, the
+//     right-hand sides in a shared-memory column that the factor takes over
+//     afterwards (190 doubles per thread: 128 threads per SM);
+//   * warp per particle (fit_warp): neighbours one per lane for the monomials,
+//     the 232 sums spread over the lanes, the factorisation and the
+//     substitutions by rows.  1.7 times the FP64 instructions, 1/20 of the
+//     latency.
+// Fits whose Jacobi-scaled conditioning estimate exceeds a threshold take one
+// corrected semi-normal-equations step (Bjorck) in the warp form: residuals
+// r_j = (U_j - U_i) - p(q_j).c are recomputed from the data, A^T W r is
+// accumulated again and solved with the same factor, so the error follows
+// cond(A) rather than cond(A^T W A) = cond(A)^2.
 #include "phb_internal.cuh"
 #include "mls_gen.cuh"
 #include "phb_mhd.cuh"
@@ -18,252 +36,695 @@
 namespace phb {
 namespace {
 
-constexpr int kT = 64;
-constexpr int kStride = kNM + kNT + kNF * kNB + 1;  // doubles per thread; odd stride avoids bank conflicts
-static_assert(4 * kNB <= kNM, "the refinement accumulates four fields in the moments' region");
+constexpr int kWarps = 4;  // per block, one block per SM: one warp per sub-partition
+constexpr int kT = 32 * kWarps;
 
-// Route queues (fits the FP32-mixed kernel handed over) up to this length
-// are fitted by a warp per particle (neighbours split over the lanes, partial
-// sums reduced in shared memory, the solve on lane 0): a handful of routed
-// fits then takes tens of microseconds instead of one thread's serial FP64
-// work.  Longer queues and the full FP64 path use one thread per particle
-// (throughput).
-constexpr int kWarpQueueMax = 4096;
+// Thread form: a warp's shared memory is [slot][32 lanes] doubles.
+constexpr int kSlots = kNT;              // the factor: 190 doubles per thread, 190 KB per block
+constexpr int kSlotOwn = kNF * kNB;      // while accumulating: x, y, z, 1/lambda, 1/r_f^2, U
+constexpr int kSlotNbr = kSlotOwn + 13;  // and two neighbours' x, y, z, U, the next one on its way
+static_assert(kSlotNbr + 2 * 11 <= kNT, "accumulators and own values must fit below the factor's end");
+
+// Warp form: per warp, doubles.
+constexpr int kRow = 39;                 // staged neighbour: w, w q^cubic (10), w dU (8), q^basis (19); odd stride
+constexpr int kWL = 32 * kRow;           // factor (packed lower triangle)
+constexpr int kWB = kWL + kNT;           // right-hand sides [field][19]
+constexpr int kWC = kWB + kNF * kNB;     // coefficients [field][19]
+constexpr int kWM = kWC + kNF * kNB;     // moments
+constexpr int kWI = kWM + kNM;           // 1 / L_kk
+constexpr int kWarpSlots = kWI + kNB;
+static_assert(kWarpSlots <= kSlots * 32, "the warp form runs in the thread form's shared memory");
+
+__device__ __forceinline__ int tri0(int r) { return r * (r + 1) / 2; }
+
+struct Box64 {
+  double len[3], inv_len[3];
+  int far[3];  // high word of a quarter box length: below it an offset is its minimum image
+};
+
+__device__ __forceinline__ Box64 make_box64(const Grid& g) {
+  Box64 b;
+  for (int c = 0; c < 3; ++c) {
+    b.len[c] = g.len[c];
+    b.inv_len[c] = g.periodic[c] ? 1.0 / g.len[c] : 0.0;
+    b.far[c] = g.periodic[c] ? __double2hiint(0.25 * g.len[c]) : 0x7fffffff;
+  }
+  return b;
+}
+
+// d - len rint(d / len) (the wrap only where it changes something)
+__device__ __forceinline__ double wrap64(const Box64& b, int c, double d) {
+  if ((__double2hiint(d) & 0x7fffffff) >= b.far[c]) d = fma(-b.len[c], rint(d * b.inv_len[c]), d);
+  return d;
+}
+
+// Squared distance over r_f^2; `inside` (s2 < 1) from the exponent bits: s2 >= 0
+// or NaN, whose high word lies above that of 1.
+__device__ __forceinline__ double dist_rel(double dx, double dy, double dz, double inv_rf2, bool& inside) {
+  const double s2 = fma(dz, dz, fma(dy, dy, __dmul_rn(dx, dx))) * inv_rf2;
+  inside = __double2hiint(s2) < 0x3ff00000;
+  return s2;
+}
+
+__device__ __forceinline__ double weight64(double s2, int weight_kind) {
+  const double sw = __dadd_rn(1.0, -s2);
+  return weight_kind == 1 ? 1.0 : __dmul_rn(sw, sw);
+}
+
+// v truncated to FP32 on the integer pipe (for the conditioning estimate).
+__device__ __forceinline__ float f32_of(double v) {
+  const unsigned hi = static_cast<unsigned>(__double2hiint(v));
+  const unsigned mag = hi & 0x7fffffffu;
+  unsigned r = __funnelshift_l(static_cast<unsigned>(__double2loint(v)), mag - 0x38000000u, 3);
+  r = mag < 0x38100000u ? 0u : (mag >= 0x47f00000u ? 0x7f7fffffu : r);
+  return __uint_as_float(r | (hi & 0x80000000u));
+}
+
+template <int N>
+struct Num {
+  static constexpr int value = N;
+};
+
+// Cholesky of columns C0 .. C0 + W - 1 of the factor in a thread's column (my,
+// stride 32), the columns before them done: the panel in registers, so that
+// its independent FMAs cover the shared-memory loads (loops of dot products
+// through shared memory took 290 cycles per FMA, this form ~90).  The diagonal
+// slots take 1 / L_kk, mkk the diagonal of M in FP32.  A Jacobi-scaled pivot
+// below 1e-12 (cond(M) above ~1e12) is treated as singular.
+template <int C0, int W>
+__device__ __forceinline__ void chol_panel(double* my, float (&mkk)[kNB], bool& singular) {
+  constexpr int R = kNB - C0;
+  double v[W][R];
+  double d[W];
+#pragma unroll
+  for (int c = 0; c < W; ++c) {
+#pragma unroll
+    for (int r = c; r < R; ++r) v[c][r] = my[(tri0(C0 + r) + C0 + c) * 32];
+    d[c] = v[c][c];
+    mkk[C0 + c] = f32_of(d[c]);
+  }
+#pragma unroll 1
+  for (int k = 0; k < C0; ++k) {
+    double l[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) l[r] = my[(tri0(C0 + r) + k) * 32];
+#pragma unroll
+    for (int c = 0; c < W; ++c)
+#pragma unroll
+      for (int r = c; r < R; ++r) v[c][r] = fma(-l[r], l[c], v[c][r]);
+  }
+#pragma unroll
+  for (int c = 0; c < W; ++c) {
+    const double p = v[c][c];
+    singular |= !(p > 0.0) || !(p > 1e-12 * d[c]);
+    const double inv = rsqrt(p > 0.0 ? p : 1.0);
+    my[(tri0(C0 + c) + C0 + c) * 32] = inv;
+#pragma unroll
+    for (int r = c + 1; r < R; ++r) {
+      v[c][r] *= inv;
+      my[(tri0(C0 + r) + C0 + c) * 32] = v[c][r];
+    }
+#pragma unroll
+    for (int e = c + 1; e < W; ++e)
+#pragma unroll
+      for (int r = e; r < R; ++r) v[e][r] = fma(-v[c][r], v[c][e], v[e][r]);
+  }
+}
+
+// Estimate of ||M_s^-1||_inf of the Jacobi-scaled matrix (as mls_inv_norm_est,
+// the back substitution by columns) in FP32 from the factor in a thread's
+// column and the diagonal mkk of M: it only picks the fits that take the
+// corrected step, and costs 700 FP64 instructions otherwise.  The factor is
+// read twice (volatile) rather than kept: 190 registers.
+__device__ __forceinline__ float inv_norm_est(const double* my, const float (&mkk)[kNB]) {
+  const volatile double* L = my;
+  float y[kNB], inv[kNB];
+#pragma unroll
+  for (int i = 0; i < kNB; ++i) {
+    float t = 0.f;
+#pragma unroll
+    for (int k = 0; k < i; ++k) t = fmaf(f32_of(L[(tri0(i) + k) * 32]), y[k], t);
+    const float sq = sqrtf(mkk[i]);
+    inv[i] = f32_of(L[(tri0(i) + i) * 32]);
+    y[i] = ((t > 0.f ? -sq : sq) - t) * inv[i];
+  }
+  float mx = 0.f;
+#pragma unroll
+  for (int k = kNB - 1; k >= 0; --k) {
+    y[k] *= inv[k];
+    mx = fmaxf(mx, fabsf(y[k]) * sqrtf(mkk[k]));
+#pragma unroll
+    for (int i = 0; i < k; ++i) y[i] = fmaf(-f32_of(L[(tri0(k) + i) * 32]), y[k], y[i]);
+  }
+  return mx;
+}
+
+// Substitutions of NF right-hand sides at once in registers, with the factor
+// in a thread's column: coefficients kQuad0 .. 18 (linear and quadratic).
+template <int NF>
+__device__ __forceinline__ void solve_thread(const double* factor, double (&b)[NF][kNB]) {
+  const volatile double* my = factor;  // read again by each group of fields rather than kept
+#pragma unroll
+  for (int i = 0; i < kNB; ++i) {
+#pragma unroll
+    for (int k = 0; k < i; ++k) {
+      const double l = my[(tri0(i) + k) * 32];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) b[f][i] = fma(-l, b[f][k], b[f][i]);
+    }
+    const double inv = my[(tri0(i) + i) * 32];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) b[f][i] *= inv;
+  }
+#pragma unroll
+  for (int i = kNB - 1; i >= kQuad0; --i) {
+#pragma unroll
+    for (int k = kNB - 1; k > i; --k) {
+      const double l = my[(tri0(k) + i) * 32];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) b[f][i] = fma(-l, b[f][k], b[f][i]);
+    }
+    const double inv = my[(tri0(i) + i) * 32];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) b[f][i] *= inv;
+  }
+}
+
+// Gradient and packed Hessian from a field's linear and quadratic coefficients.
+template <class C>
+__device__ __forceinline__ void derivs_of(C c, double il, double il2, double (&g)[3], double (&h)[6]) {
+  for (int k = 0; k < 3; ++k) g[k] = c(kLin0 + k) * il;
+  h[0] = 2.0 * c(kQuad0) * il2;
+  h[1] = c(kQuad0 + 1) * il2;
+  h[2] = c(kQuad0 + 2) * il2;
+  h[3] = 2.0 * c(kQuad0 + 3) * il2;
+  h[4] = c(kQuad0 + 4) * il2;
+  h[5] = 2.0 * c(kQuad0 + 5) * il2;
+}
+
+__device__ __forceinline__ void write_derivs(const FitArgs& a, int f, int dst, const double (&g)[3],
+                                             const double (&h)[6]) {
+  const int64_t n = a.n;
+  for (int c = 0; c < 3; ++c) a.grad[(f * 3 + c) * n + dst] = g[c];
+  if (a.hess)
+    for (int c = 0; c < 6; ++c) a.hess[(f * 6 + c) * n + dst] = h[c];
+}
+
+// Time derivatives of slot s.  Out of line: both forms then run the same code.
+__device__ __noinline__ void write_rhs(const FitArgs& a, int s, int dst, const MhdDerivs<double>& D) {
+  const int64_t n = a.n;
+  double u[8];
+  for (int f = 0; f < 8; ++f) u[f] = a.sU[f * n + s];
+  const int src = a.perm_in ? a.perm_in[s] : s;
+  double zeta = a.zeta ? a.zeta[src] : 0.0;
+  double eta = a.eta ? a.eta[src] : 0.0;
+  if (a.c_zeta_l != 0.0 || a.c_zeta_a != 0.0 || a.c_eta != 0.0)
+    mhd_laws(u, D, a.gamma, a.slam[s], a.c_zeta_l, a.c_zeta_a, a.c_eta, zeta, eta);
+  double out[8];
+  mhd_rhs(u, D, a.gamma, zeta, eta, out);
+  bool finite = true;
+  for (int f = 0; f < 8; ++f) {
+    finite &= finite64(out[f]);
+    a.dudt[f * n + dst] = out[f];
+  }
+  if (!finite) raise_flag(a.status_word, PHB_FLAG_NONFINITE);
+}
+
+__device__ __forceinline__ int64_t list_end(const FitArgs& a, int s) {
+  const int64_t e = a.off[s + 1];
+  return e < a.g.capacity ? e : a.g.capacity;
+}
+
+// One particle per lane (slot < 0: none); my: the lane's shared-memory column
+// (stride 32).  All lanes call it, and the lanes meet again after every
+// neighbour: left to themselves the lanes of lists of different lengths ran
+// the loop apart, in up to twice the time.  Returns true, with nothing
+// written, when the fit needs the corrected step.
+template <FitMode MODE>
+__device__ __forceinline__ bool fit_thread(const FitArgs& a, const Box64& bx, int slot, bool routed,
+                                           float refine_above, double* my) {
+  constexpr int f0 = MODE == FitMode::kRHS ? 1 : 0;  // the RHS never needs the density fit
+  const int64_t n = a.n;
+  const int s = slot < 0 ? 0 : slot;
+  const double lam = a.slam[s];
+  const double inv_l = 1.0 / lam;
+  const int64_t beg = a.off[s];
+  const int len = slot < 0 ? 0 : static_cast<int>(list_end(a, s) - beg);
+  const int longest = __reduce_max_sync(0xffffffffu, len);
+  // the particle's own values in shared memory, read when used: registers
+  // hold the 80 moments
+  volatile double* own = my + kSlotOwn * 32;
+  {
+    const double rf = a.g.rf_factor * lam;
+    for (int c = 0; c < 3; ++c) own[c * 32] = a.spos[c * n + s];
+    own[3 * 32] = inv_l;
+    own[4 * 32] = 1.0 / (rf * rf);
+    for (int f = f0; f < kNF; ++f) own[(5 + f) * 32] = a.sU[f * n + s];
+  }
+  for (int k = f0 * kNB; k < kNF * kNB; ++k) my[k * 32] = 0.0;
+  double m[kNM];
+#pragma unroll
+  for (int k = 0; k < kNM; ++k) m[k] = 0.0;
+  int cnt = 0;
+  // the next neighbour's values are copied to shared memory during this one's
+  // sums (no registers, and their latency, ~1,400 cycles a neighbour, hidden)
+  constexpr int kNbr = 3 + kNF - f0;
+  volatile double* nbr = my + kSlotNbr * 32;
+  auto fetch = [&](int t, int e) {
+    const unsigned to = static_cast<unsigned>(__cvta_generic_to_shared(my + (kSlotNbr + (e & 1) * kNbr) * 32));
+#pragma unroll
+    for (int c = 0; c < kNbr; ++c) {
+      const double* from = c < 3 ? a.spos + c * n + t : a.sU + (f0 + c - 3) * n + t;
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(to + c * 256), "l"(from) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int32_t* list = a.idx + beg;
+  fetch(len > 0 ? list[0] : s, 0);
+  int next = len > 1 ? list[1] : s;
+#pragma unroll 1
+  for (int e = 0; e < longest; ++e) {
+    fetch(next, e + 1);
+    next = e + 2 < len ? list[e + 2] : s;
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    const volatile double* at = nbr + (e & 1) * kNbr * 32;
+    const double dx = wrap64(bx, 0, at[0] - own[0]);
+    const double dy = wrap64(bx, 1, at[32] - own[32]);
+    const double dz = wrap64(bx, 2, at[64] - own[64]);
+    bool inside;
+    const double s2 = dist_rel(dx, dy, dz, own[4 * 32], inside);
+    if (inside && e < len) {
+      ++cnt;
+      const double wt = weight64(s2, a.weight_kind);
+      double qg[kNB], wq[kNB + 1];
+      const double il = own[3 * 32];
+      mls_monomials_cubic_w(dx * il, dy * il, dz * il, wt, qg, wq);
+      // the sums in shared memory are loaded two ahead: with the moments in
+      // registers the compiler otherwise loads each just before its FMA
+      // (123 instead of 70 cycles per FMA)
+      volatile double* b = my + f0 * kNB * 32;
+      constexpr int N = (kNF - f0) * kNB;
+      double ahead[2] = {b[0], b[32]};
+#pragma unroll
+      for (int f = f0; f < kNF; ++f) {
+        const double wdu = wt * (at[(3 + f - f0) * 32] - own[(5 + f) * 32]);
+#pragma unroll
+        for (int k = 0; k < kNB; ++k) {
+          const int i = (f - f0) * kNB + k;
+          const double v = ahead[i & 1];
+          if (i + 2 < N) ahead[i & 1] = b[(i + 2) * 32];
+          b[i * 32] = fma(qg[k], wdu, v);
+        }
+      }
+      mls_accum_moments(qg, wq, m);
+    }
+    __syncwarp();
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  // the right-hand sides to local memory, the normal matrix in their place
+  double b[kNF * kNB];
+#pragma unroll 4
+  for (int k = f0 * kNB; k < kNF * kNB; ++k) b[k] = my[k * 32];
+  struct Col {
+    double* p;
+    __device__ __forceinline__ double& operator[](int k) const { return p[k * 32]; }
+  };
+  Col M{my};
+  mls_assemble(m, M);
+  bool singular = cnt < kNB;
+  if (!singular) {
+    float mkk[kNB];
+    chol_panel<0, 4>(my, mkk, singular);
+    chol_panel<4, 4>(my, mkk, singular);
+    chol_panel<8, 5>(my, mkk, singular);
+    chol_panel<13, 6>(my, mkk, singular);
+    if (!singular && kNB * inv_norm_est(my, mkk) > refine_above) return true;
+  }
+  if (slot < 0) return false;
+  const int dst = a.perm_out ? a.perm_out[s] : s;
+  if (a.fit_status) a.fit_status[dst] = singular ? 1 : (routed ? 2 : 0);
+  if (singular) raise_flag(a.status_word, PHB_FLAG_FIT_SINGULAR);
+  const double il2 = inv_l * inv_l;
+  MhdDerivs<double> D;
+  mhd_zero(D);
+  // fields f .. f + N - 1
+  auto fields = [&](int f, auto group) {
+    constexpr int N = decltype(group)::value;
+    double c[N][kNB];
+#pragma unroll
+    for (int u = 0; u < N; ++u)
+#pragma unroll
+      for (int k = 0; k < kNB; ++k) c[u][k] = b[(f + u) * kNB + k];
+    solve_thread(my, c);
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      double g[3] = {0, 0, 0}, h[6] = {0, 0, 0, 0, 0, 0};
+      if (!singular) derivs_of([&](int k) { return c[u][k]; }, inv_l, il2, g, h);
+      if (MODE == FitMode::kDerivs) write_derivs(a, f + u, dst, g, h);
+      else mhd_collect(D, f + u, g, h);
+    }
+  };
+  if (MODE == FitMode::kDerivs) {
+#pragma unroll 1
+    for (int f = 0; f < kNF; f += 4) fields(f, Num<4>{});
+  } else {
+    fields(1, Num<4>{});
+    fields(5, Num<3>{});
+    write_rhs(a, s, dst, D);
+  }
+  return false;
+}
+
+// What a lane does in the warp form: its sums (operands within a staged
+// neighbour's row) and its entries of the normal matrix.
+struct WarpTab {
+  int sum[8];    // byte offsets: first | second << 16
+  int entry[6];  // row | column << 8 | moment << 16; column -1 (0xff): none
+};
 
 template <FitMode MODE>
-__global__ void __launch_bounds__(kT, 1) k_fit_fp64(const FitArgs a, int routed, const int32_t* list,
-                                                 const int32_t* list_len) {
+__device__ __forceinline__ void warp_tab(WarpTab& w, int lane) {
+  constexpr int f0 = MODE == FitMode::kRHS ? 1 : 0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int t = lane + 32 * u;
+    int x = 0, y = 0;
+    if (t < kNM) {
+      mls_moment_split(t, x, y);
+      y += kNB;
+    } else if (t < kNM + (kNF - f0) * kNB) {
+      x = 11 + f0 + (t - kNM) / kNB;
+      y = kNB + (t - kNM) % kNB;
+    }
+    w.sum[u] = x * 8 | (y * 8) << 16;
+  }
+  // entries from the bottom right corner, column by column: those right of
+  // column j are a prefix
+#pragma unroll
+  for (int u = 0; u < 6; ++u) {
+    const int t = lane + 32 * u;
+    int k = 0;
+    while (tri0(k + 1) <= t) ++k;
+    const int col = kNB - 1 - k, row = kNB - 1 - (t - tri0(k));
+    w.entry[u] = t < kNT ? row | col << 8 | mls_moment_index(row, col) << 16 : 0xff00;
+  }
+}
+
+// Sums over the neighbours of slot s; with Res, of the residuals of the
+// coefficients in W[kWC..] instead of the field differences.  Moments to
+// W[kWM..], right-hand sides to W[kWB..].  Returns the neighbours within r_f.
+template <FitMode MODE, bool Res>
+__device__ __forceinline__ int warp_sums(const FitArgs& a, const Box64& bx, const WarpTab& tab, int s,
+                                         double inv_l, double inv_rf2, double* W, int lane) {
+  constexpr int f0 = MODE == FitMode::kRHS ? 1 : 0;
+  constexpr int nsum = kNM + (kNF - f0) * kNB;
+  constexpr int rounds = (nsum + 31) / 32;
+  const int64_t n = a.n;
+  const int64_t beg = a.off[s], end = list_end(a, s);
+  const double xs = a.spos[s], ys = a.spos[n + s], zs = a.spos[2 * n + s];
+  double acc[rounds];
+#pragma unroll
+  for (int u = 0; u < rounds; ++u) acc[u] = 0.0;
+  int cnt = 0;
+  for (int64_t c0 = beg; c0 < end; c0 += 32) {
+    const int64_t e = c0 + lane;
+    bool inside = false;
+    double dx = 0, dy = 0, dz = 0, s2 = 0;
+    double du[kNF];
+    if (e < end) {
+      const int t = a.idx[e];
+#pragma unroll
+      for (int f = f0; f < kNF; ++f) du[f] = a.sU[f * n + t] - a.sU[f * n + s];
+      dx = wrap64(bx, 0, a.spos[t] - xs);
+      dy = wrap64(bx, 1, a.spos[n + t] - ys);
+      dz = wrap64(bx, 2, a.spos[2 * n + t] - zs);
+      s2 = dist_rel(dx, dy, dz, inv_rf2, inside);
+    }
+    const unsigned in = __ballot_sync(0xffffffffu, inside);
+    if (inside) {
+      double* row = W + __popc(in & ((1u << lane) - 1u)) * kRow;
+      const double wt = weight64(s2, a.weight_kind);
+      double qg[kNB], wq[kNB + 1];
+      mls_monomials_cubic_w(dx * inv_l, dy * inv_l, dz * inv_l, wt, qg, wq);
+#pragma unroll
+      for (int k = 0; k < 11; ++k) row[k] = wq[k];
+#pragma unroll
+      for (int k = 0; k < kNB; ++k) row[kNB + k] = qg[k];
+#pragma unroll
+      for (int f = f0; f < kNF; ++f) {
+        double r = du[f];
+        if (Res)
+#pragma unroll
+          for (int k = 0; k < kNB; ++k) r = fma(-qg[k], W[kWC + f * kNB + k], r);
+        row[11 + f] = wt * r;
+      }
+    }
+    __syncwarp();
+    const int m = __popc(in);
+    cnt += m;
+    const char* row = reinterpret_cast<const char*>(W);
+#pragma unroll 2
+    for (int j = 0; j < m; ++j, row += kRow * 8)
+#pragma unroll
+      for (int u = 0; u < rounds; ++u)
+        acc[u] = fma(*reinterpret_cast<const double*>(row + (tab.sum[u] & 0xffff)),
+                     *reinterpret_cast<const double*>(row + (tab.sum[u] >> 16)), acc[u]);
+    __syncwarp();
+  }
+#pragma unroll
+  for (int u = 0; u < rounds; ++u) {
+    const int t = lane + 32 * u;
+    if (t < kNM) W[kWM + t] = acc[u];
+    else if (t < nsum) W[kWB + f0 * kNB + t - kNM] = acc[u];
+  }
+  __syncwarp();
+  return cnt;
+}
+
+// inv_norm_est with a row per lane (each sum in its order).
+__device__ __forceinline__ float warp_inv_norm_est(const double* W, int lane) {
+  const double* L = W + kWL;
+  const int i = lane < kNB ? lane : kNB - 1;
+  const float inv = f32_of(W[kWI + i]);
+  const float sq = sqrtf(f32_of(W[kWM + mls_moment_index(i, i)]));
+  float s = 0.f, y = 0.f;
+#pragma unroll
+  for (int k = 0; k < kNB; ++k) {
+    if (lane == k) y = ((s > 0.f ? -sq : sq) - s) * inv;
+    const float yk = __shfl_sync(0xffffffffu, y, k);
+    if (i > k) s = fmaf(f32_of(L[tri0(i) + k]), yk, s);
+  }
+#pragma unroll
+  for (int k = kNB - 1; k >= 0; --k) {
+    if (lane == k) y *= inv;
+    const float xk = __shfl_sync(0xffffffffu, y, k);
+    if (i < k) y = fmaf(-f32_of(L[tri0(k) + i]), xk, y);
+  }
+  const float x = lane < kNB ? fabsf(y) * sq : 0.f;
+  return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));
+}
+
+// Substitutions of all fields at once, four lanes per field (rows i = q mod 4);
+// coefficients Lo .. 18 of each field to v (row q + 4 u).
+template <int Lo>
+__device__ __forceinline__ void warp_solve(const double* W, const double* rhs, int q, double (&v)[5]) {
+  const double* L = W + kWL;
+  const double* inv = W + kWI;
+#pragma unroll
+  for (int u = 0; u < 5; ++u) v[u] = q + 4 * u < kNB ? rhs[q + 4 * u] : 0.0;
+#pragma unroll
+  for (int k = 0; k < kNB; ++k) {
+    const double y = __shfl_sync(0xffffffffu, v[k >> 2] * inv[k], k & 3, 4);
+    if (q == (k & 3)) v[k >> 2] = y;
+#pragma unroll
+    for (int u = 0; u < 5; ++u) {
+      const int i = q + 4 * u;
+      if (4 * u + 3 > k && i > k && i < kNB) v[u] = fma(-L[tri0(i) + k], y, v[u]);
+    }
+  }
+#pragma unroll
+  for (int i = kNB - 1; i >= Lo; --i) {
+    const double c = __shfl_sync(0xffffffffu, v[i >> 2] * inv[i], i & 3, 4);
+    if (q == (i & 3)) v[i >> 2] = c;
+#pragma unroll
+    for (int u = 0; u < 5; ++u) {
+      const int k = q + 4 * u;
+      if (4 * u < i && 4 * u + 3 >= Lo && k >= Lo && k < i) v[u] = fma(-L[tri0(i) + k], c, v[u]);
+    }
+  }
+}
+
+// One particle by one warp (all lanes call it with the same s).
+template <FitMode MODE>
+__device__ __forceinline__ void fit_warp(const FitArgs& a, const Box64& bx, const WarpTab& tab, int s,
+                                         bool routed, float refine_above, double* W) {
+  constexpr int f0 = MODE == FitMode::kRHS ? 1 : 0;
+  const int lane = threadIdx.x & 31;
+  const double lam = a.slam[s];
+  const double rf = a.g.rf_factor * lam;
+  const double inv_l = 1.0 / lam, inv_rf2 = 1.0 / (rf * rf);
+  const int cnt = warp_sums<MODE, false>(a, bx, tab, s, inv_l, inv_rf2, W, lane);
+  bool singular = cnt < kNB;
+  double* L = W + kWL;
+  const int q = lane & 3, f = f0 + (lane >> 2);
+  const bool mine = f < kNF;
+  if (!singular) {
+    // each lane keeps its entries of the matrix; per column: the owners write
+    // it out, every lane forms 1 / L_jj, the rows below are scaled, and the
+    // entries right of it are updated
+    double e[6];
+    int row[6], col[6];
+#pragma unroll
+    for (int u = 0; u < 6; ++u) {
+      row[u] = tab.entry[u] & 0xff;
+      col[u] = tab.entry[u] >> 8 & 0xff;
+      e[u] = W[kWM + (tab.entry[u] >> 16)];
+      if (row[u] == col[u]) W[kWI + row[u]] = e[u];  // M_jj until 1 / L_jj takes its place
+    }
+#pragma unroll 1
+    for (int j = 0; j < kNB; ++j) {
+#pragma unroll
+      for (int u = 0; u < 6; ++u)
+        if (col[u] == j) L[tri0(row[u]) + j] = e[u];
+      __syncwarp();
+      const double p = L[tri0(j) + j], d = W[kWI + j];
+      const int below = tri0(j + 1 + lane) + j;
+      const double v = j + 1 + lane < kNB ? L[below] : 0.0;
+      singular |= !(p > 0.0) || !(p > 1e-12 * d);
+      const double r = rsqrt(p > 0.0 ? p : 1.0);
+      if (j + 1 + lane < kNB) L[below] = v * r;
+      __syncwarp();
+      if (lane == 0) W[kWI + j] = r;
+#pragma unroll
+      for (int u = 0; u < 6; ++u)
+        if (col[u] > j && col[u] < kNB)
+          e[u] = fma(-L[tri0(row[u]) + j], L[tri0(col[u]) + j], e[u]);
+    }
+    __syncwarp();
+  }
+  bool refine = false;
+  if (!singular) {
+    const float est = warp_inv_norm_est(W, lane);
+    refine = kNB * est > refine_above;
+    __syncwarp();
+    double v[5];
+    const double* rhs = W + kWB + (mine ? f : f0) * kNB;
+    if (refine) {
+      warp_solve<0>(W, rhs, q, v);
+      if (mine)
+#pragma unroll
+        for (int u = 0; u < 5; ++u)
+          if (q + 4 * u < kNB) W[kWC + f * kNB + q + 4 * u] = v[u];
+      __syncwarp();
+      warp_sums<MODE, true>(a, bx, tab, s, inv_l, inv_rf2, W, lane);
+      warp_solve<kQuad0>(W, rhs, q, v);
+      if (mine)
+#pragma unroll
+        for (int u = 2; u < 5; ++u)
+          if (q + 4 * u >= kQuad0 && q + 4 * u < kNB) W[kWC + f * kNB + q + 4 * u] += v[u];
+    } else {
+      warp_solve<kQuad0>(W, rhs, q, v);
+      if (mine)
+#pragma unroll
+        for (int u = 2; u < 5; ++u)
+          if (q + 4 * u < kNB) W[kWC + f * kNB + q + 4 * u] = v[u];
+    }
+  }
+  __syncwarp();
+  const int dst = a.perm_out ? a.perm_out[s] : s;
+  const double il2 = inv_l * inv_l;
+  if (lane == 0) {
+    if (a.fit_status) a.fit_status[dst] = singular ? 1 : (routed ? 2 : 0);
+    if (singular) raise_flag(a.status_word, PHB_FLAG_FIT_SINGULAR);
+  }
+  if (MODE == FitMode::kDerivs) {
+    if (q == 0) {
+      double g[3] = {0, 0, 0}, h[6] = {0, 0, 0, 0, 0, 0};
+      if (!singular) derivs_of([&](int k) { return W[kWC + f * kNB + k]; }, inv_l, il2, g, h);
+      write_derivs(a, f, dst, g, h);
+    }
+  } else if (lane == 0) {
+    MhdDerivs<double> D;
+    mhd_zero(D);
+#pragma unroll
+    for (int k = f0; k < kNF; ++k) {
+      double g[3] = {0, 0, 0}, h[6] = {0, 0, 0, 0, 0, 0};
+      if (!singular) derivs_of([&](int c) { return W[kWC + k * kNB + c]; }, inv_l, il2, g, h);
+      mhd_collect(D, k, g, h);
+    }
+    write_rhs(a, s, dst, D);
+  }
+  __syncwarp();  // the next particle takes the same shared memory
+}
+
+// Which form serves which part of the work: a pass of the thread form over
+// the grid fits gridDim x 128 particles (19,456 on 152 SMs) in 0.65 ms
+// whatever their number, the warp form gridDim x 4 particles in 34 us; so
+// full passes go to the thread form and a remainder of up to kWarpPasses
+// passes of the warp form (0.54 ms) to the warp form.
+constexpr int kWarpPasses = 8;
+
+// Particles: the slots of `list` (device count *list_len), or all, taken tile
+// by tile in the order of tmap (longest lists first within a tile), so that
+// a warp's loops are of similar length.
+template <FitMode MODE>
+__global__ void __launch_bounds__(kT, 1) k_fit_fp64(const __grid_constant__ FitArgs a, bool routed,
+                                                    const int32_t* list, const int32_t* list_len,
+                                                    const uint8_t* tmap) {
   extern __shared__ double sm[];
-  const int n = a.n;
-  const int total = list ? *list_len : n;
-  // uniform over the launch; an active subset in FP64 keeps one thread per
-  // particle so that its results are bit-identical to the full evaluation
-  const int lanes = (routed && list && total <= kWarpQueueMax) ? 32 : 1;
+  const int total = list ? *list_len : static_cast<int>((a.n + a.g.tile - 1) / a.g.tile) * a.g.tile;
+  const int pass = gridDim.x * kT, warp_pass = gridDim.x * kWarps;
+  int full = total / pass * pass;
+  if (total - full > kWarpPasses * warp_pass) full = total;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // warps numbered across the SMs first: a last, partial pass spreads over them
+  const int gw = wid * gridDim.x + blockIdx.x;
+  if (full == 0 && gw >= total) return;  // an empty or short queue: no FP64 set-up
+  const Box64 bx = make_box64(a.g);
+  double* W = sm + wid * kSlots * 32;
   // fits routed from the FP32-mixed path need ~1e-5: FP64 normal equations
   // meet that up to cond(M) ~ 1e9; the FP64 path itself targets ~1e-12
-  const double refine_above = routed ? 1e9 : 1e4;
-  const int lane = threadIdx.x % lanes;
-  const int groups = kT / lanes;
-  const int grp = threadIdx.x / lanes;
-  // a block without work (an empty or short routed queue) leaves before any
-  // FP64 set-up
-  if (static_cast<int64_t>(blockIdx.x) * groups >= total) return;
-  double* my = sm + threadIdx.x * kStride;
-  double* head = sm + grp * lanes * kStride;  // the group's lane 0 region: totals, factor, c
-  double(&mom)[kNM] = *reinterpret_cast<double(*)[kNM]>(my);
-  double(&M)[kNT] = *reinterpret_cast<double(*)[kNT]>(head + kNM);
-  double* bs = my + kNM + kNT;
-  double* hmom = head;
-  double* hbs = head + kNM + kNT;
-  constexpr int f0 = MODE == FitMode::kRHS ? 1 : 0;  // the RHS never needs the density fit
-  // fields fitted, in U order without rho for the RHS
-  double len[3], inv_len[3];
-  for (int c = 0; c < 3; ++c) {
-    len[c] = a.g.len[c];
-    inv_len[c] = a.g.periodic[c] ? 1.0 / a.g.len[c] : 0.0;
-  }
-  // sum the lanes' partial accumulators [0, count) of the regions starting at
-  // `at` into the group's lane 0 region (no-op for one lane per particle)
-  auto reduce = [&](int at, int count) {
-    if (lanes == 1) return;
-    __syncwarp();
-    for (int k = lane; k < count; k += lanes) {
-      double t = 0.0;
-      for (int l = 0; l < lanes; ++l) t += head[l * kStride + at + k];
-      head[at + k] = t;
-    }
-    __syncwarp();
+  const float refine_above = routed ? 1e9f : 1e4f;
+  auto slot = [&](int w) {
+    if (list) return w < total ? list[w] : -1;
+    if (w >= total) return -1;
+    const int s = w / a.g.tile * a.g.tile + tmap[w];
+    return s < a.n ? s : -1;
   };
-  for (int w = blockIdx.x * groups + grp; w < total; w += gridDim.x * groups) {
-    const int s = list ? list[w] : w;
-    const double xs = a.spos[s], ys = a.spos[n + s], zs = a.spos[2 * n + s];
-    double u[8];
-#pragma unroll
-    for (int f = 0; f < 8; ++f) u[f] = a.sU[f * static_cast<int64_t>(n) + s];
-    const double lam = a.slam[s];
-    const double rf = a.g.rf_factor * lam;
-    const double inv_rf2 = 1.0 / (rf * rf);
-    const double inv_l = 1.0 / lam;
-    const int64_t beg = a.off[s];
-    const int64_t end = a.off[s + 1] < a.g.capacity ? a.off[s + 1] : a.g.capacity;
-    for (int k = 0; k < kNM; ++k) mom[k] = 0.0;
-    for (int k = 0; k < kNF * kNB; ++k) bs[k] = 0.0;
-    int cnt = 0;
-    for (int64_t e = beg + lane; e < end; e += lanes) {
-      const int t = a.idx[e];
-      double dx = a.spos[t] - xs, dy = a.spos[n + t] - ys, dz = a.spos[2 * n + t] - zs;
-      dx -= len[0] * rint(dx * inv_len[0]);
-      dy -= len[1] * rint(dy * inv_len[1]);
-      dz -= len[2] * rint(dz * inv_len[2]);
-      const double s2 = (dx * dx + dy * dy + dz * dz) * inv_rf2;
-      const bool inside = s2 < 1.0;
-      if (!inside) continue;
-      ++cnt;
-      const double sw = 1.0 - s2;
-      const double wt = a.weight_kind == 1 ? 1.0 : sw * sw;
-      double qg[kNB], wq[kNB + 1];
-      mls_monomials(dx * inv_l, dy * inv_l, dz * inv_l, wt, qg, wq);
-      mls_accum_moments(qg, wq, mom);
-#pragma unroll
-      for (int f = f0; f < kNF; ++f) {
-        const double du = a.sU[f * static_cast<int64_t>(n) + t] - u[f];
-        mls_accum_rhs(wq, du, *reinterpret_cast<double(*)[kNB]>(bs + f * kNB));
-      }
+  for (int w0 = gw * 32; w0 < full; w0 += pass) {
+    const int s = w0 + lane < full ? slot(w0 + lane) : -1;
+    const bool refine = fit_thread<MODE>(a, bx, s, routed, refine_above, W + lane);
+    __syncwarp();
+    unsigned todo = __ballot_sync(0xffffffffu, refine);
+    if (todo != 0u) {
+      WarpTab tab;
+      warp_tab<MODE>(tab, lane);
+      for (; todo != 0u; todo &= todo - 1u)
+        fit_warp<MODE>(a, bx, tab, __shfl_sync(0xffffffffu, s, __ffs(todo) - 1), routed, refine_above, W);
     }
-    if (lanes > 1) cnt = __reduce_add_sync(0xffffffffu, cnt);
-    reduce(0, kNM);                      // moments
-    reduce(kNM + kNT, kNF * kNB);        // right-hand sides
-    bool singular = cnt < kNB;
-    bool refine = false;
-    double invd[kNB];
-    if (lane == 0 && !singular) {
-      mls_assemble(*reinterpret_cast<double(*)[kNM]>(hmom), M);
-      const double minpiv = mls_cholesky<double>(M, invd);
-      double rmin = 1e300;
-#pragma unroll
-      for (int k = 0; k < kNB; ++k) {
-        const double r = 1.0 / (invd[k] * invd[k] * M[k * (k + 1) / 2 + k]);
-        rmin = r < rmin ? r : rmin;
-      }
-      // a Jacobi-scaled pivot below 1e-12 (cond(M) above ~1e12) is treated as singular
-      singular = !(minpiv > 0.0) || !(rmin > 1e-12);
-      // normal equations lose cond(M) * eps: above an estimate of refine_above
-      // (n_b times the greedy ||M_s^-1||_inf estimate) take one corrected
-      // semi-normal-equations step (residuals recomputed from the data)
-      refine = !singular && kNB * mls_inv_norm_est<double>(M, invd) > refine_above;
-      if (lanes > 1)
-        for (int k = 0; k < kNB; ++k) head[kStride + k] = invd[k];  // lane 1's region is free here
+  }
+  if (full + gw < total) {
+    WarpTab tab;
+    warp_tab<MODE>(tab, lane);
+    for (int w = full + gw; w < total; w += warp_pass) {
+      const int s = slot(w);
+      if (s >= 0) fit_warp<MODE>(a, bx, tab, s, routed, refine_above, W);
     }
-    if (lanes > 1) {
-      singular = __shfl_sync(0xffffffffu, singular, 0);
-      refine = __shfl_sync(0xffffffffu, refine, 0);
-      __syncwarp();
-      if (lane > 0 && lane < kNF - f0 && !singular)
-        for (int k = 0; k < kNB; ++k) invd[k] = head[kStride + k];
-      __syncwarp();
-    }
-    // coefficients of every field: the linear and quadratic ones, or all 19
-    // when the fit is refined; kept in the right-hand-side region.  One lane
-    // per field with a warp per particle, all fields in turn otherwise.
-    const int fstep = lanes > 1 ? kNF : 1;
-    if (!singular) {
-      for (int f = f0 + (lanes > 1 ? lane : 0); f < kNF; f += fstep) {
-        double b[kNB];
-#pragma unroll
-        for (int j = 0; j < kNB; ++j) b[j] = hbs[f * kNB + j];
-        mls_forward(M, invd, b);
-        if (refine) mls_back19(M, invd, b);
-        else mls_back9(M, invd, b);
-#pragma unroll
-        for (int j = 0; j < kNB; ++j) hbs[f * kNB + j] = b[j];
-      }
-    }
-    if (lanes > 1) __syncwarp();
-    const int dst = a.perm_out ? a.perm_out[s] : s;
-    if (refine) {
-      // corrected semi-normal equations: one pass over the neighbours per
-      // group of up to four fields accumulates A^T W r with the residuals
-      // r = (U_j - U_i) - p(q_j).c recomputed from the data; the moments'
-      // region (dead after the assembly) holds the four accumulators
-      for (int g0 = f0; g0 < kNF; g0 += 4) {
-        const int g1 = g0 + 4 < kNF ? g0 + 4 : kNF;
-        for (int k = 0; k < 4 * kNB; ++k) mom[k] = 0.0;
-        for (int64_t e = beg + lane; e < end; e += lanes) {
-          const int t = a.idx[e];
-          double dx = a.spos[t] - xs, dy = a.spos[n + t] - ys, dz = a.spos[2 * n + t] - zs;
-          dx -= len[0] * rint(dx * inv_len[0]);
-          dy -= len[1] * rint(dy * inv_len[1]);
-          dz -= len[2] * rint(dz * inv_len[2]);
-          const double s2 = (dx * dx + dy * dy + dz * dz) * inv_rf2;
-          if (!(s2 < 1.0)) continue;
-          const double sw = 1.0 - s2;
-          const double wt = a.weight_kind == 1 ? 1.0 : sw * sw;
-          double qg[kNB], wq[kNB + 1];
-          mls_monomials(dx * inv_l, dy * inv_l, dz * inv_l, wt, qg, wq);
-          for (int f = g0; f < g1; ++f) {
-            double r = a.sU[f * static_cast<int64_t>(n) + t] - u[f];
-#pragma unroll
-            for (int k = 0; k < kNB; ++k) r = fma(-qg[k], hbs[f * kNB + k], r);
-            mls_accum_rhs(wq, r, *reinterpret_cast<double(*)[kNB]>(mom + (f - g0) * kNB));
-          }
-        }
-        reduce(0, 4 * kNB);
-        for (int f = g0 + (lanes > 1 ? lane : 0); f < g1; f += fstep) {
-          double acc[kNB];
-#pragma unroll
-          for (int k = 0; k < kNB; ++k) acc[k] = hmom[(f - g0) * kNB + k];
-          mls_forward(M, invd, acc);
-          mls_back9(M, invd, acc);
-#pragma unroll
-          for (int k = kQuad0; k < kNB; ++k) hbs[f * kNB + k] += acc[k];
-        }
-        if (lanes > 1) __syncwarp();
-      }
-    }
-    if (lane == 0) {
-      if (a.fit_status) a.fit_status[dst] = singular ? 1 : (routed ? 2 : 0);
-      if (singular) raise_flag(a.status_word, PHB_FLAG_FIT_SINGULAR);
-      const double il = inv_l, il2 = inv_l * inv_l;
-      MhdDerivs<double> D;
-      mhd_zero(D);
-      for (int f = f0; f < kNF; ++f) {
-        double g[3] = {0, 0, 0}, h[6] = {0, 0, 0, 0, 0, 0};
-        if (!singular) {
-          const double* b = hbs + f * kNB;
-          g[0] = b[kLin0] * il; g[1] = b[kLin0 + 1] * il; g[2] = b[kLin0 + 2] * il;
-          h[0] = 2.0 * b[kQuad0] * il2; h[1] = b[kQuad0 + 1] * il2; h[2] = b[kQuad0 + 2] * il2;
-          h[3] = 2.0 * b[kQuad0 + 3] * il2; h[4] = b[kQuad0 + 4] * il2; h[5] = 2.0 * b[kQuad0 + 5] * il2;
-        }
-        if (MODE == FitMode::kDerivs) {
-          for (int c = 0; c < 3; ++c) a.grad[(f * 3 + c) * static_cast<int64_t>(n) + dst] = g[c];
-          if (a.hess)
-            for (int c = 0; c < 6; ++c) a.hess[(f * 6 + c) * static_cast<int64_t>(n) + dst] = h[c];
-        } else {
-          mhd_collect(D, f, g, h);
-        }
-      }
-      if (MODE == FitMode::kRHS) {
-        const int src = a.perm_in ? a.perm_in[s] : s;
-        double zeta = a.zeta ? a.zeta[src] : 0.0;
-        double eta = a.eta ? a.eta[src] : 0.0;
-        if (a.c_zeta_l != 0.0 || a.c_zeta_a != 0.0 || a.c_eta != 0.0)
-          mhd_laws(u, D, a.gamma, lam, a.c_zeta_l, a.c_zeta_a, a.c_eta, zeta, eta);
-        double out[8];
-        mhd_rhs(u, D, a.gamma, zeta, eta, out);
-        bool finite = true;
-        for (int f = 0; f < 8; ++f) {
-          finite &= isfinite(out[f]);
-          a.dudt[f * static_cast<int64_t>(n) + dst] = out[f];
-        }
-        if (!finite) raise_flag(a.status_word, PHB_FLAG_NONFINITE);
-      }
-    }
-    if (lanes > 1) __syncwarp();  // the group's regions are reused by the next particle
   }
 }
 
 }  // namespace
 
 cudaError_t launch_fit_fp64(const FitArgs& a, FitMode mode, const int32_t* list,
-                            const int32_t* list_len, cudaStream_t st, bool routed) {
-  const size_t smem = size_t(kStride) * kT * sizeof(double);
-  unsigned blocks = list ? static_cast<unsigned>(num_sms() * 2)
-                         : static_cast<unsigned>((a.n + kT - 1) / kT);
-  if (mode == FitMode::kDerivs) {
-    cudaFuncSetAttribute(k_fit_fp64<FitMode::kDerivs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(smem));
-    const int tr = trace_begin(list ? 3 : 2, st);
-    k_fit_fp64<FitMode::kDerivs><<<blocks, kT, smem, st>>>(a, routed, list, list_len);
-    note_launch();
-    trace_end(tr, st);
-  } else {
-    cudaFuncSetAttribute(k_fit_fp64<FitMode::kRHS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(smem));
-    const int tr = trace_begin(list ? 3 : 2, st);
-    k_fit_fp64<FitMode::kRHS><<<blocks, kT, smem, st>>>(a, routed, list, list_len);
-    note_launch();
-    trace_end(tr, st);
-  }
+                            const int32_t* list_len, const uint8_t* tmap, cudaStream_t st, bool routed) {
+  const size_t smem = size_t(kSlots) * kT * sizeof(double);
+  const unsigned blocks = static_cast<unsigned>(num_sms());
+  const auto kernel = mode == FitMode::kDerivs ? k_fit_fp64<FitMode::kDerivs> : k_fit_fp64<FitMode::kRHS>;
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const int tr = trace_begin(list ? 3 : 2, st);
+  kernel<<<blocks, kT, smem, st>>>(a, routed, list, list_len, tmap);
+  note_launch();
+  trace_end(tr, st);
   return cudaGetLastError();
 }
 

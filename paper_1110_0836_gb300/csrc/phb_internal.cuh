@@ -451,10 +451,12 @@ FitArgs fit_args(const phb_plan* plan, const phb_params* prm, void* ws, const in
                  double* dudt, double* grad, double* hess, int32_t* fit_status,
                  int32_t* status_word);
 
-// FP64 fused fit over all slots (list == null) or over list[0 .. *list_len);
-// routed: the list is the FP32-mixed kernel's route queue (fit status 2).
+// FP64 fused fit over all slots (list == null; tmap: the build's order of each
+// tile's particles) or over list[0 .. *list_len); routed: the list is the
+// FP32-mixed kernel's route queue (fit status 2).
 cudaError_t launch_fit_fp64(const FitArgs& a, FitMode mode, const int32_t* list,
-                            const int32_t* list_len, cudaStream_t st, bool routed = false);
+                            const int32_t* list_len, const uint8_t* tmap, cudaStream_t st,
+                            bool routed = false);
 int num_sms();
 size_t l2_bytes();  // L2 cache size of the current device (queried once)
 

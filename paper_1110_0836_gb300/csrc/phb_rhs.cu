@@ -158,17 +158,17 @@ cudaError_t run_fit(const phb_plan* plan, const phb_params* prm, void* ws, FitMo
     a.pc_h = hu->h;
   }
   cudaError_t e;
-  if (prm->precision == PHB_FP64) return launch_fit_fp64(a, mode, list, list_len, st);
+  const uint8_t* tmap = region<uint8_t>(plan, ws, R_TMAP);
+  if (prm->precision == PHB_FP64) return launch_fit_fp64(a, mode, list, list_len, tmap, st);
   if ((e = cudaMemsetAsync(a.queue_len, 0, sizeof(int32_t), st))) return e;
   if ((e = cudaMemsetAsync(a.queue_len + 2, 0, sizeof(int32_t), st))) return e;
   if ((e = cudaMemsetAsync(a.refined_tiles, 0, 2 * sizeof(int32_t), st))) return e;  // and rq_len
   if ((e = launch_fit_mixed(a, mode, region<int2>(plan, ws, R_TPLAN), region<int32_t>(plan, ws, R_TSLOT),
-                            region<uint16_t>(plan, ws, R_LSELF), region<uint8_t>(plan, ws, R_TMAP),
-                            region<uint16_t>(plan, ws, R_LIDX),
+                            region<uint16_t>(plan, ws, R_LSELF), tmap, region<uint16_t>(plan, ws, R_LIDX),
                             a.queue_len + 2,
                             region<int32_t>(plan, ws, R_TORDER), list, list_len, list_cap, st)))
     return e;
-  return launch_fit_fp64(a, mode, a.queue, a.queue_len, st, true);
+  return launch_fit_fp64(a, mode, a.queue, a.queue_len, tmap, st, true);
 }
 
 }  // namespace phb
