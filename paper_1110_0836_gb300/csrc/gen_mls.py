@@ -433,56 +433,54 @@ def gen():
             w(f"    y[{i}] = __fmul2_rn(v, make_float2(inv_diag[{i}], inv_diag[{i}])); }}")
         w("}")
         w("")
-    # ---- adjoint helpers: all monomials of degree 0..6 and polynomial gradients
-    MONO = sorted({(a, b, c) for a in range(7) for b in range(7) for c in range(7) if a + b + c <= 6},
-                  key=lambda e: (sum(e), [-x for x in e]))
-    assert len(MONO) == 84
-    MO = {e: i for i, e in enumerate(MONO)}
-    w("constexpr int kNMono = 84;  // monomials of total degree 0..6")
-    w("")
-    w("// All monomials q^a of total degree 0..6 (graded order, mono[0] = 1).")
-    w("template <typename T>")
-    w("__device__ __forceinline__ void mls_monos6(T x, T y, T z, T (&mono)[kNMono]) {")
-    w("  mono[0] = T(1);")
-    for e in MONO[1:]:
-        # build from a lower monomial times one coordinate
-        for ax, nm in ((0, "x"), (1, "y"), (2, "z")):
-            if e[ax] > 0:
-                lower = list(e); lower[ax] -= 1
-                w(f"  mono[{MO[e]}] = mono[{MO[tuple(lower)]}] * {nm};  // {name(e)}")
-                break
-    w("}")
-    w("")
-    w("// P = sum_alpha mbar[alpha] q^alpha over the 80 moments and its gradient in q.")
+    # ---- adjoint helpers
+    # nested (Horner) evaluation of sum_alpha mbar[alpha] q^alpha + sum_beta B[beta] p_beta(q)
+    # and its gradient: in z inside y inside x, each level with the derivative
+    # recurrence d <- d t + v, v <- v t + c.  199 multiply-adds and 16 additions,
+    # against 430 with the 84 monomials tabulated.
+    w("// P = sum_alpha mbar[alpha] q^alpha (80 moments) + sum_beta B[beta] p_beta(q) (19 basis")
+    w("// monomials) and its gradient in q, by nested multiplication.")
     w("template <typename T, typename MB>")
-    w("__device__ __forceinline__ void mls_eval_moment_poly(const T (&mono)[kNMono], const MB& mbar, T& P, T& Px, T& Py, T& Pz) {")
-    w("  T p = T(0), px = T(0), py = T(0), pz = T(0);")
-    for a, al in enumerate(MOMENTS):
-        w(f"  {{ const T c = mbar[{a}];")
-        w(f"    p = fma(c, mono[{MO[al]}], p);")
-        for ax, acc in ((0, "px"), (1, "py"), (2, "pz")):
-            if al[ax] > 0:
-                lo = list(al); lo[ax] -= 1
-                coef = f"T({al[ax]}) * " if al[ax] > 1 else ""
-                w(f"    {acc} = fma({coef}c, mono[{MO[tuple(lo)]}], {acc});")
-        w("  }")
+    w("__device__ __forceinline__ void mls_poly_grad(T x, T y, T z, const MB& mbar, const T (&B)[kNB], T& P, T& Px, T& Py, T& Pz) {")
+
+    def coef(e):
+        d = sum(e)
+        if d == 1:
+            return f"B[{IDX[e]}]"
+        if d <= 3:
+            return f"(mbar[{MIDX[e]}] + B[{IDX[e]}])"
+        return f"mbar[{MIDX[e]}]"
+
+    def step(v, t, c):  # v <- v t + c
+        return f"fma({v}, {t}, {c})" if c is not None else f"{v} * {t}"
+    w("  T p, px, py, pz, q, qy, qz, r, rz;")
+    for i in range(6, -1, -1):
+        for j in range(6 - i, -1, -1):
+            d = 6 - i - j
+            # R_ij(z) and its derivative
+            w(f"  r = {coef((i, j, d))};")
+            for k in range(d - 1, -1, -1):
+                if k == d - 1:
+                    w("  rz = r;")
+                else:
+                    w("  rz = fma(rz, z, r);")
+                c = coef((i, j, k)) if i + j + k > 0 else None
+                w(f"  r = {step('r', 'z', c)};")
+            # Q_i(y, z) = sum_j y^j R_ij
+            if d == 0:
+                w("  q = r;")
+            else:
+                w("  qy = q;" if d == 1 else "  qy = fma(qy, y, q);")
+                w("  qz = rz;" if d == 1 else "  qz = fma(qz, y, rz);")
+                w("  q = fma(q, y, r);")
+        if i == 6:
+            w("  p = q;")
+        else:
+            w("  px = p;" if i == 5 else "  px = fma(px, x, p);")
+            w("  py = qy;" if i == 5 else "  py = fma(py, x, qy);")
+            w("  pz = qz;" if i == 5 else "  pz = fma(pz, x, qz);")
+            w("  p = fma(p, x, q);")
     w("  P = p; Px = px; Py = py; Pz = pz;")
-    w("}")
-    w("")
-    w("// V = sum_beta B[beta] p_beta(q) over the 19 basis monomials and its gradient in q.")
-    w("template <typename T, typename BB>")
-    w("__device__ __forceinline__ void mls_eval_basis_poly(const T (&mono)[kNMono], const BB& B, T& V, T& Vx, T& Vy, T& Vz) {")
-    w("  T v = T(0), vx = T(0), vy = T(0), vz = T(0);")
-    for i, be in enumerate(BASIS):
-        w(f"  {{ const T c = B[{i}];")
-        w(f"    v = fma(c, mono[{MO[be]}], v);")
-        for ax, acc in ((0, "vx"), (1, "vy"), (2, "vz")):
-            if be[ax] > 0:
-                lo = list(be); lo[ax] -= 1
-                coef = f"T({be[ax]}) * " if be[ax] > 1 else ""
-                w(f"    {acc} = fma({coef}c, mono[{MO[tuple(lo)]}], {acc});")
-        w("  }")
-    w("  V = v; Vx = vx; Vy = vy; Vz = vz;")
     w("}")
     w("")
     w("// Adjoint of the normal matrix through its moments:")
@@ -494,18 +492,6 @@ def gen():
             w(f"  mbar[{MIDX[add(BASIS[r], BASIS[cc])]}] = fma(-bbar[{r}], c[{cc}], mbar[{MIDX[add(BASIS[r], BASIS[cc])]}]);")
     w("}")
     w("")
-    w("// The 19 basis values from the monomial table.")
-    w("template <typename T>")
-    w("__device__ __forceinline__ void mls_basis_from_monos(const T (&mono)[kNMono], T (&p)[kNB]) {")
-    for i, be in enumerate(BASIS):
-        w(f"  p[{i}] = mono[{MO[be]}];")
-    w("}")
-    w("")
-    w("// Basis value p_beta(q) from the monomial table.")
-    w("__device__ __forceinline__ int mls_basis_mono(int i) {")
-    w("  constexpr unsigned char t[kNB] = {" + ", ".join(str(MO[b]) for b in BASIS) + "};")
-    w("  return t[i];")
-    w("}")
     w("}  // namespace phb")
     return "\n".join(L) + "\n"
 

@@ -14,54 +14,56 @@
 //               qbar_j   = w_j grad_q[ sum_a mbar_a q^a + sum_f dU_fj p(q) . bbar_f ]
 //               dbar_j   = qbar_j / lambda_i + wbar_j dw/dd,
 //             whose negatives are particle i's own terms (U_i, x_i).
-// The first kernel keeps, per particle, only its adjoint seeds bbar_f and
-// mbar (213 doubles) and its own terms; a second kernel gathers, for every
-// particle j, the contributions of each i that lists j - through a reverse
-// neighbour list in ascending order of i, recomputing q, w, p(q) and dw/dd
-// of the entry from the positions - so the result does not depend on thread
-// scheduling and no per-entry buffer is needed.  By default the factorisation is
-// recomputed here (nothing is stored by the forward call); the stored variant
-// records, per particle, the Cholesky factor, its Jacobi scaling and the
-// fitted coefficients once (kRecord) and the adjoint then starts from that
-// record (kStored) instead of re-accumulating the moments and right-hand sides.
-#include "phb_internal.cuh"
-#include "mls_gen.cuh"
+// k_adjoint takes a particle per thread through all of it: the fit as in
+// phb_fit64.cuh, the seeds bbar_f and mbar in the shared memory that held the
+// factor, then the neighbours, whose ten terms go to a buffer, one row per
+// list entry.  k_adj_gather sums, for every particle j, the rows of the entries
+// that name it, through a reverse list in ascending order of the entries, so
+// the result does not depend on thread scheduling.  The buffer holds a bounded
+// part of the entries: the particles are taken in chunks of consecutive slots.
+//
+// What bounds it: the FP64 pipe (see phb_fit_fp64.cu).  Per neighbour the fit
+// takes 267 FP64 instructions and the backward pass ~500 (2 x 7 x 19 products
+// with the seeds, 180 for the degree-6 polynomial and its gradient by nested
+// multiplication); forming every entry's terms once and passing them through
+// memory (80 B written and read per entry, 0.3 ms per 262,144 particles) costs
+// less than forming them a second time for the neighbour.  Four warps per SM
+// (213 doubles of shared memory per thread).  Measured, 262,144 particles:
+// gradient 62.4 -> 30.0 ms (before: each entry's terms formed again in the gather, 84
+// tabulated monomials, seeds in global memory).
+//
+// By default the factorisation is recomputed here (nothing is stored by the
+// forward call); the stored variant records, per particle, the Cholesky
+// factor, its diagonal's reciprocals and the fitted coefficients once
+// (kRecord) and the adjoint then starts from that record (kStored) instead of
+// re-accumulating the moments and right-hand sides.
+#include "phb_fit64.cuh"
 #include "phb_mhd.cuh"
 
 namespace phb {
 namespace {
 
-constexpr int kT = 64;
+constexpr int kWarps = 4;  // per block, one block per SM: one warp per sub-partition
+constexpr int kT = 32 * kWarps;
 constexpr int kThreads = 256;
-constexpr int kNFit = 7;                 // fitted fields: U indices 1..7 (V, B, sigma)
-constexpr int kSm = kNM + kNFit * kNB;   // 213 doubles per thread (the 190-entry M overlays it)
-// per-particle scratch record (contiguous per particle, read by the gather):
-// bbar_f (7 x 19), then the coefficients c_f (7 x 19) of the recomputing
-// form, whose first 80 words take mbar once c_f is no longer needed
-constexpr int kScrBbar = 0, kScrC = kNFit * kNB, kScrMbar = kScrC, kScr = 2 * kNFit * kNB;
-static_assert(kSm >= kNT, "shared region must hold the normal matrix");
-// record of one particle's forward fit, [k][n] layout: factor (190), Jacobi
-// scaling invd (19), coefficients c_f (7 x 19), then 1 = singular / 0 = regular
+constexpr int kNFit = 7;  // fitted fields: U indices 1..7 (V, B, sigma)
+// a lane's column: the fit, the factor, then bbar_f [field][19] and mbar [80]
+constexpr int kSlotMbar = kNFit * kNB;
+constexpr int kSlots = kSlotMbar + kNM;
+static_assert(kSlots >= kNT && size_t(kSlots) * kT * 8 <= 227 * 1024, "shared memory of a block");
+// record of one particle's forward fit, [k][n] layout: factor (190, 1 / L_kk on
+// its diagonal), 1 / L_kk (19), coefficients c_f (7 x 19), then 1 = singular /
+// 0 = regular
 constexpr int kRecFac = 0, kRecInvd = kNT, kRecCoef = kNT + kNB, kRecFlag = kRecCoef + kNFit * kNB;
 constexpr int kRecWords = kRecFlag + 1;
+constexpr int kTerms = 10;  // an entry's row: dUbar of fields 1..7, dbar
 enum AdjMode { kRecompute = 0, kRecord = 1, kStored = 2 };
-
-// Column view of thread-private shared memory ([k][kT] layout, no bank conflicts).
-struct SCol {
-  double* p;
-  __device__ __forceinline__ double& operator[](int k) const { return p[k * kT]; }
-};
-// Column view of a per-particle array in global scratch ([k][n] layout, coalesced).
-struct GCol {
-  double* p;
-  int64_t n;
-  __device__ __forceinline__ double& operator[](int k) const { return p[k * n]; }
-};
 
 struct AdjArgs {
   Grid g;
   int32_t n;
   const int32_t* perm;   // slot -> caller index
+  const uint8_t* tmap;   // per tile: its particles, longest list first
   const double* spos;
   const double* slam;
   const double* sU;
@@ -73,29 +75,36 @@ struct AdjArgs {
   const double* zeta;    // caller order or null
   const double* eta;
   double c_zeta_l, c_zeta_a, c_eta;  // coefficient laws (phb_params), 0 = off
-  double* scr;           // [n][kScr] slot order: bbar_f, then c_f / mbar
-  double* self;          // [11][n] slot order
+  double* terms;         // [entries of a chunk][kTerms]
+  double* acc;           // [11][n] slot order: Ubar, xbar so far
   double* rec;           // [kRecWords][n] slot order (stored variant) or null
   int32_t* status_word;
+  int64_t span;          // list entries per chunk (rows of `terms` less n)
+  int32_t chunk, chunks;
 };
 
-struct Geo {
-  double dx, dy, dz, s2;
-};
+// First slot whose list starts at entry e0 or later (a warp samples 32 points
+// per step).
+__device__ __forceinline__ int first_slot(const int64_t* off, int n, int64_t e0) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, hi = n;  // off[lo - 1] < e0 <= off[hi]
+  while (lo < hi) {
+    const int step = (hi - lo + 31) / 32;
+    const int at = lo + lane * step;
+    const unsigned below = __ballot_sync(0xffffffffu, at < hi && off[at] < e0);
+    if (below == 0u) return lo;
+    const int last = lo + (31 - __clz(below)) * step;  // off[last] < e0
+    lo = last + 1;
+    hi = min(hi, last + step);
+  }
+  return lo;
+}
 
-__device__ __forceinline__ Geo geometry(const AdjArgs& a, int t, double xs, double ys, double zs,
-                                        const double (&len)[3], const double (&ilen)[3],
-                                        double inv_rf2) {
-  const int64_t N = a.n;
-  Geo q;
-  q.dx = a.spos[t] - xs;
-  q.dy = a.spos[N + t] - ys;
-  q.dz = a.spos[2 * N + t] - zs;
-  q.dx -= len[0] * rint(q.dx * ilen[0]);
-  q.dy -= len[1] * rint(q.dy * ilen[1]);
-  q.dz -= len[2] * rint(q.dz * ilen[2]);
-  q.s2 = (q.dx * q.dx + q.dy * q.dy + q.dz * q.dz) * inv_rf2;
-  return q;
+// Slots [first, last) of the chunk: those whose lists start in its span of the
+// entries (a list is shorter than n, so their entries fit span + n rows).
+__device__ __forceinline__ void chunk_slots(const AdjArgs& a, int& first, int& last) {
+  first = a.chunk == 0 ? 0 : first_slot(a.off, a.n, a.chunk * a.span);
+  last = a.chunk == a.chunks - 1 ? a.n : first_slot(a.off, a.n, (a.chunk + 1) * a.span);
 }
 
 // Adjoint of the right-hand side at one particle.  In: point values u, the
@@ -188,310 +197,338 @@ __device__ void rhs_adjoint_point(const double (&u)[8], const MhdDerivs<double>&
   gb[3 + 0][1] -= Jb[2];
 }
 
-// Adjoint contribution of one list entry (particle i at xs with fields u,
-// neighbour t) to the neighbour: ub[f] to U_t (fitted fields 1..7) and xb to
-// x_t, from i's seeds bbar_f (stride bs) and mbar (stride ms).  The entry's
-// offset, weight, monomials and dw/dd are recomputed from the positions.
-// Returns false (nothing written) for an entry beyond r_f,i (skin).
-__device__ __forceinline__ bool entry_adjoint(const AdjArgs& a, int t, double xs, double ys,
-                                              double zs, const double (&u)[8], double inv_rf2,
-                                              double inv_l, const double (&len)[3],
-                                              const double (&ilen)[3], const double* bb, int bs,
-                                              const double* mbar, int ms, double (&ub)[kNFit],
-                                              double (&xb)[3]) {
-  const int64_t N = a.n;
-  const Geo q = geometry(a, t, xs, ys, zs, len, ilen, inv_rf2);
-  if (!(q.s2 < 1.0)) return false;
-  const double sw = 1.0 - q.s2;
-  const double wt = a.weight_kind == 1 ? 1.0 : sw * sw;
-  double mono[kNMono];
-  mls_monos6(q.dx * inv_l, q.dy * inv_l, q.dz * inv_l, mono);
-  double p[kNB];
-  mls_basis_from_monos(mono, p);
-  double Bt[kNB];
-  for (int k = 0; k < kNB; ++k) Bt[k] = 0.0;
-  for (int fi = 0; fi < kNFit; ++fi) {
-    const double du = a.sU[(fi + 1) * N + t] - u[fi + 1];
-    double pb = 0.0;
-    for (int k = 0; k < kNB; ++k) {
-      const double bk = bb[(fi * kNB + k) * bs];
-      pb = fma(p[k], bk, pb);
-      Bt[k] = fma(du, bk, Bt[k]);
-    }
-    ub[fi] = wt * pb;
-  }
-  struct Strided {
-    const double* p;
-    int st;
-    __device__ __forceinline__ double operator[](int k) const { return p[k * st]; }
-  };
-  double V, Vx, Vy, Vz, P, Px, Py, Pz;
-  mls_eval_basis_poly(mono, Bt, V, Vx, Vy, Vz);
-  mls_eval_moment_poly(mono, Strided{mbar, ms}, P, Px, Py, Pz);
-  const double wbar = P + V;
-  const double dwd_c = a.weight_kind == 1 ? 0.0 : -4.0 * inv_rf2;
-  const double dw = wbar * dwd_c * sw;  // d w / d d = -4 (1 - s^2) d / r_f^2
-  xb[0] = wt * (Px + Vx) * inv_l + dw * q.dx;
-  xb[1] = wt * (Py + Vy) * inv_l + dw * q.dy;
-  xb[2] = wt * (Pz + Vz) * inv_l + dw * q.dz;
-  return true;
-}
-
 template <int MODE>
-__global__ void __launch_bounds__(kT, 1) k_adjoint(const AdjArgs a) {
+__global__ void __launch_bounds__(kT, 1) k_adjoint(const __grid_constant__ AdjArgs a) {
   extern __shared__ double sm[];
-  const int s = blockIdx.x * kT + threadIdx.x;
-  if (s >= a.n) return;
-  double* my = sm + threadIdx.x;
-  const SCol M{my};                 // normal matrix / factor (190), later mbar (80) + bbar (133)
-  const SCol MB{my};                // mbar [80]
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double* my = sm + wid * kSlots * 32 + lane;
   const int64_t N = a.n;
-  // c_f, f = 0..6: [f * 19 + k] (in the record for the stored variant)
-  double* my_scr = a.scr + static_cast<int64_t>(s) * kScr;
-  const GCol cf{MODE == kRecompute ? my_scr + kScrC : a.rec + kRecCoef * N + s,
-                MODE == kRecompute ? 1 : N};
-  const GCol bbar{my_scr + kScrBbar, 1};          // bbar_f
-  double len[3], ilen[3];
-  for (int c = 0; c < 3; ++c) {
-    len[c] = a.g.len[c];
-    ilen[c] = a.g.periodic[c] ? 1.0 / a.g.len[c] : 0.0;
-  }
-  const double xs = a.spos[s], ys = a.spos[N + s], zs = a.spos[2 * N + s];
-  double u[8];
-  for (int f = 0; f < 8; ++f) u[f] = a.sU[f * N + s];
-  const double lam = a.slam[s];
-  const double rf = a.g.rf_factor * lam;
-  const double inv_rf2 = 1.0 / (rf * rf);
-  const double inv_l = 1.0 / lam;
-  const int64_t beg = a.off[s];
-  const int64_t end = a.off[s + 1] < a.g.capacity ? a.off[s + 1] : a.g.capacity;
-  const int src = a.perm[s];
-  const double zeta = a.zeta ? a.zeta[src] : 0.0;
-  const double eta = a.eta ? a.eta[src] : 0.0;
-
-  // ---- forward: moments
-  int cnt = 0;
-  double invd[kNB];
-  bool singular;
-  if (MODE == kStored) {
-    singular = a.rec[kRecFlag * N + s] != 0.0;
-    if (!singular) {
-      for (int k = 0; k < kNT; ++k) M[k] = a.rec[(kRecFac + k) * N + s];
-      for (int k = 0; k < kNB; ++k) invd[k] = a.rec[(kRecInvd + k) * N + s];
-    }
-  } else {
-    double m[kNM];
+  int first = 0, last = a.n;
+  if (MODE != kRecord) chunk_slots(a, first, last);
+  if (first >= last) return;
+  const int64_t row0 = MODE == kRecord ? 0 : a.off[first];
+  const Box64 bx = make_box64(a.g);
+  const int T = a.g.tile;
+  const int w_end = (last + T - 1) / T * T;
+  // warps numbered across the SMs first: a last, partial pass spreads over them
+  for (int w0 = first / T * T + (wid * gridDim.x + blockIdx.x) * 32; w0 < w_end; w0 += gridDim.x * kT) {
+    const int own = w0 / T * T + a.tmap[w0 + lane];
+    const bool act = own >= first && own < last;
+    const int s = act ? own : first;
+    const double lam = a.slam[s];
+    const double rf = a.g.rf_factor * lam;
+    const double inv_rf2 = 1.0 / (rf * rf), il = 1.0 / lam, il2 = il * il;
+    const int64_t beg = a.off[s];
+    const int len = act ? list_len64(a.off, a.g.capacity, s) : 0;
+    double c[kNFit * kNB];  // right-hand sides, then coefficients c_f
+    bool singular;
+    if (MODE == kStored) {
+      singular = a.rec[kRecFlag * N + s] != 0.0;
+      if (!singular) {
+#pragma unroll 10
+        for (int k = 0; k < kNT; ++k) my[k * 32] = a.rec[(kRecFac + k) * N + s];
+#pragma unroll 10
+        for (int k = 0; k < kNFit * kNB; ++k) c[k] = a.rec[(kRecCoef + k) * N + s];
+      }
+    } else {
+      double m[kNM];
+      const int cnt = accum_thread<1>(a.spos, a.sU, N, a.idx + beg, len, s, bx, a.weight_kind, il,
+                                      inv_rf2, my, m);
+#pragma unroll 4
+      for (int k = 0; k < kNFit * kNB; ++k) c[k] = my[(kNB + k) * 32];
+      struct Col {
+        double* p;
+        __device__ __forceinline__ double& operator[](int k) const { return p[k * 32]; }
+      };
+      Col M{my};
+      mls_assemble(m, M);
+      singular = cnt < kNB;
+      if (!singular) {
+        float mkk[kNB];
+        chol_panel<0, 4>(my, mkk, singular);
+        chol_panel<4, 4>(my, mkk, singular);
+        chol_panel<8, 5>(my, mkk, singular);
+        chol_panel<13, 6>(my, mkk, singular);
+      }
+      if (!singular) {
+        auto solve = [&](int f, auto group) {
+          constexpr int G = decltype(group)::value;
+          double b[G][kNB];
 #pragma unroll
-    for (int k = 0; k < kNM; ++k) m[k] = 0.0;
-    for (int64_t e = beg; e < end; ++e) {
-      const Geo q = geometry(a, a.idx[e], xs, ys, zs, len, ilen, inv_rf2);
-      if (!(q.s2 < 1.0)) continue;
-      ++cnt;
-      const double sw = 1.0 - q.s2;
-      const double wt = a.weight_kind == 1 ? 1.0 : sw * sw;
-      double qg[kNB], wq[kNB + 1];
-      mls_monomials(q.dx * inv_l, q.dy * inv_l, q.dz * inv_l, wt, qg, wq);
-      mls_accum_moments(qg, wq, m);
-    }
-    singular = cnt < kNB;
-    if (!singular) mls_assemble(m, M);
-  }
-  if (MODE != kStored && !singular) {
-    const double minpiv = mls_cholesky<double>(M, invd);
-    double rmin = 1e300;
-    for (int k = 0; k < kNB; ++k) {
-      const double r = 1.0 / (invd[k] * invd[k] * M[k * (k + 1) / 2 + k]);
-      rmin = r < rmin ? r : rmin;
-    }
-    singular = !(minpiv > 0.0) || !(rmin > 1e-12);
-  }
-  if (MODE == kRecord) {
-    a.rec[kRecFlag * N + s] = singular ? 1.0 : 0.0;
-    if (singular) {
-      raise_flag(a.status_word, PHB_FLAG_FIT_SINGULAR);
-      return;
-    }
-    for (int k = 0; k < kNT; ++k) a.rec[(kRecFac + k) * N + s] = M[k];
-    for (int k = 0; k < kNB; ++k) a.rec[(kRecInvd + k) * N + s] = invd[k];
-  }
-  double selfu[8], selfx[3] = {0.0, 0.0, 0.0};
-  if (singular) {
-    // the forward right-hand side is zero and does not depend on the inputs:
-    // no own terms and zero seeds for the gather
-    for (int k = 0; k < kNFit * kNB; ++k) my_scr[kScrBbar + k] = 0.0;
-    for (int k = 0; k < kNM; ++k) my_scr[kScrMbar + k] = 0.0;
-    for (int k = 0; k < 11; ++k) a.self[k * N + s] = 0.0;
-    raise_flag(a.status_word, PHB_FLAG_FIT_SINGULAR);
-    return;
-  }
-  // ---- forward: right-hand sides in two groups, full coefficients c_f
-  for (int grp = 0; grp < (MODE == kStored ? 0 : 2); ++grp) {
-    const int nf = grp == 0 ? 4 : 3;  // fields 1..4 (Vx, Vy, Vz, Bx) then 5..7 (By, Bz, sigma)
-    double b[4][kNB];
-    for (int f = 0; f < 4; ++f)
-      for (int k = 0; k < kNB; ++k) b[f][k] = 0.0;
-    for (int64_t e = beg; e < end; ++e) {
-      const int t = a.idx[e];
-      const Geo q = geometry(a, t, xs, ys, zs, len, ilen, inv_rf2);
-      if (!(q.s2 < 1.0)) continue;
-      const double sw = 1.0 - q.s2;
-      const double wt = a.weight_kind == 1 ? 1.0 : sw * sw;
-      double qg[kNB], wq[kNB + 1];
-      mls_monomials(q.dx * inv_l, q.dy * inv_l, q.dz * inv_l, wt, qg, wq);
-      for (int f = 0; f < nf; ++f) {
-        const int uf = 1 + grp * 4 + f;
-        mls_accum_rhs(wq, a.sU[uf * N + t] - u[uf], b[f]);
+          for (int u = 0; u < G; ++u)
+#pragma unroll
+            for (int k = 0; k < kNB; ++k) b[u][k] = c[(f + u) * kNB + k];
+          solve_thread<G, 0, 0>(my, b);
+#pragma unroll
+          for (int u = 0; u < G; ++u)
+#pragma unroll
+            for (int k = 0; k < kNB; ++k) c[(f + u) * kNB + k] = b[u][k];
+        };
+        solve(0, Num<4>{});
+        solve(4, Num<3>{});
       }
     }
-    for (int f = 0; f < nf; ++f) {
-      mls_forward(M, invd, b[f]);
-      mls_back19(M, invd, b[f]);
-      const int fi = grp * 4 + f;  // 0..6 <-> U index 1..7
-      for (int k = 0; k < kNB; ++k) cf[fi * kNB + k] = b[f][k];
-    }
-  }
-  if (MODE == kRecord) return;
-  double o[8];
-  for (int f = 0; f < 8; ++f) o[f] = a.gbar[f * N + src];
-  // ---- derivatives, right-hand-side adjoint, cbar -> bbar = M^-1 cbar
-  const double il = inv_l, il2 = inv_l * inv_l;
-  {
-    MhdDerivs<double> D;
-    mhd_zero(D);
-    for (int fi = 0; fi < kNFit; ++fi) {
-      const double g[3] = {cf[fi * kNB + kLin0] * il, cf[fi * kNB + kLin0 + 1] * il,
-                           cf[fi * kNB + kLin0 + 2] * il};
-      const double h[6] = {2.0 * cf[fi * kNB + kQuad0] * il2, cf[fi * kNB + kQuad0 + 1] * il2,
-                           cf[fi * kNB + kQuad0 + 2] * il2, 2.0 * cf[fi * kNB + kQuad0 + 3] * il2,
-                           cf[fi * kNB + kQuad0 + 4] * il2, 2.0 * cf[fi * kNB + kQuad0 + 5] * il2};
-      mhd_collect(D, fi + 1, g, h);
-    }
-    double gb[kNFit][3], hb[kNFit][6];
-    rhs_adjoint_point(u, D, a.gamma, zeta, eta, lam, a.c_zeta_l, a.c_zeta_a, a.c_eta, o, selfu,
-                      gb, hb);
-    for (int fi = 0; fi < kNFit; ++fi) {
-      double cb[kNB];
-      for (int k = 0; k < kQuad0; ++k) cb[k] = 0.0;
-      cb[kQuad0] = 2.0 * hb[fi][0] * il2;
-      cb[kQuad0 + 1] = hb[fi][1] * il2;
-      cb[kQuad0 + 2] = hb[fi][2] * il2;
-      cb[kQuad0 + 3] = 2.0 * hb[fi][3] * il2;
-      cb[kQuad0 + 4] = hb[fi][4] * il2;
-      cb[kQuad0 + 5] = 2.0 * hb[fi][5] * il2;
-      cb[kLin0] = gb[fi][0] * il;
-      cb[kLin0 + 1] = gb[fi][1] * il;
-      cb[kLin0 + 2] = gb[fi][2] * il;
-      mls_forward(M, invd, cb);
-      mls_back19(M, invd, cb);
-      for (int k = 0; k < kNB; ++k) bbar[fi * kNB + k] = cb[k];
-    }
-  }
-  // ---- mbar = fold of -sum_f bbar_f c_f^T onto the moments; stage mbar, bbar
-  // in shared memory and keep mbar in the scratch record (over c_f) for the gather
-  {
-    double mb[kNM];
-#pragma unroll
-    for (int k = 0; k < kNM; ++k) mb[k] = 0.0;
-    for (int fi = 0; fi < kNFit; ++fi) {
-      double bb[kNB], cc[kNB];
-      for (int k = 0; k < kNB; ++k) {
-        bb[k] = bbar[fi * kNB + k];
-        cc[k] = cf[fi * kNB + k];
+    if (act && singular) raise_flag(a.status_word, PHB_FLAG_FIT_SINGULAR);
+    if (MODE == kRecord) {
+      if (act) {
+        a.rec[kRecFlag * N + s] = singular ? 1.0 : 0.0;
+        if (!singular) {
+#pragma unroll 10
+          for (int k = 0; k < kNT; ++k) a.rec[(kRecFac + k) * N + s] = my[k * 32];
+          for (int k = 0; k < kNB; ++k) a.rec[(kRecInvd + k) * N + s] = my[(tri0(k) + k) * 32];
+#pragma unroll 10
+          for (int k = 0; k < kNFit * kNB; ++k) a.rec[(kRecCoef + k) * N + s] = c[k];
+        }
       }
-      mls_accum_mbar(bb, cc, mb);
-    }
-#pragma unroll
-    for (int k = 0; k < kNM; ++k) {
-      MB[k] = mb[k];
-      my_scr[kScrMbar + k] = mb[k];
-    }
-    for (int k = 0; k < kNFit * kNB; ++k) M[kNM + k] = bbar[k];  // M is dead now
-  }
-  // ---- backward pass over the neighbours: particle i's own terms
-  for (int64_t e = beg; e < end; ++e) {
-    const int t = a.idx[e];
-    double ub[kNFit], xb[3];
-    if (!entry_adjoint(a, t, xs, ys, zs, u, inv_rf2, inv_l, len, ilen, M.p + kNM * kT, kT,
-                       MB.p, kT, ub, xb))
+      __syncwarp();
       continue;
-    for (int fi = 0; fi < kNFit; ++fi) selfu[fi + 1] -= ub[fi];
-    for (int c = 0; c < 3; ++c) selfx[c] -= xb[c];
-  }
-  for (int k = 0; k < 8; ++k) a.self[k * N + s] = selfu[k];
-  for (int c = 0; c < 3; ++c) a.self[(8 + c) * N + s] = selfx[c];
-}
-
-// ---- reverse neighbour lists: for every particle t, the particles i whose
-// list names t, in ascending order of i
-__global__ void k_rev_count(int n, int64_t cap, const int64_t* __restrict__ off,
-                            const int32_t* __restrict__ idx, int32_t* __restrict__ rcnt) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int64_t end = off[i + 1] < cap ? off[i + 1] : cap;
-  for (int64_t e = off[i]; e < end; ++e) atomicAdd(&rcnt[idx[e]], 1);
-}
-
-__global__ void k_rev_fill(int n, int64_t cap, const int64_t* __restrict__ off,
-                           const int32_t* __restrict__ idx, const int64_t* __restrict__ roff,
-                           int32_t* __restrict__ rcur, int32_t* __restrict__ rsrc) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int64_t end = off[i + 1] < cap ? off[i + 1] : cap;
-  for (int64_t e = off[i]; e < end; ++e) {
-    const int t = idx[e];
-    rsrc[roff[t] + atomicAdd(&rcur[t], 1)] = i;
-  }
-}
-
-__global__ void k_rev_sort(int n, const int64_t* __restrict__ roff, int32_t* __restrict__ rsrc) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  int32_t* v = rsrc + roff[t];
-  const int m = static_cast<int>(roff[t + 1] - roff[t]);
-  for (int i = 1; i < m; ++i) {
-    const int32_t x = v[i];
-    int j = i - 1;
-    while (j >= 0 && v[j] > x) {
-      v[j + 1] = v[j];
-      --j;
     }
-    v[j + 1] = x;
+    // a singular fit's right-hand side is zero and does not depend on the
+    // inputs: no own terms, and zero rows for the gather
+    const bool live = act && !singular;
+    double u[8], selfu[8], selfx[3] = {0.0, 0.0, 0.0};
+    for (int f = 0; f < 8; ++f) {
+      u[f] = a.sU[f * N + s];
+      selfu[f] = 0.0;
+    }
+    if (live) {
+      const int src = a.perm[s];
+      double o[8];
+      for (int f = 0; f < 8; ++f) o[f] = a.gbar[f * N + src];
+      // derivatives, right-hand-side adjoint, cbar -> bbar = M^-1 cbar
+      double bbar[kNFit * kNB];
+      {
+        MhdDerivs<double> D;
+        mhd_zero(D);
+#pragma unroll
+        for (int f = 0; f < kNFit; ++f) {
+          double g[3], h[6];
+          derivs_of([&](int k) { return c[f * kNB + k]; }, il, il2, g, h);
+          mhd_collect(D, f + 1, g, h);
+        }
+        double gb[kNFit][3], hb[kNFit][6];
+        rhs_adjoint_point(u, D, a.gamma, a.zeta ? a.zeta[src] : 0.0, a.eta ? a.eta[src] : 0.0, lam,
+                          a.c_zeta_l, a.c_zeta_a, a.c_eta, o, selfu, gb, hb);
+        auto seeds = [&](auto from, auto group) {
+          constexpr int F = decltype(from)::value, G = decltype(group)::value;
+          double b[G][kNB];
+#pragma unroll
+          for (int v = 0; v < G; ++v) {
+#pragma unroll
+            for (int k = 0; k < kQuad0; ++k) b[v][k] = 0.0;
+            b[v][kQuad0] = 2.0 * hb[F + v][0] * il2;
+            b[v][kQuad0 + 1] = hb[F + v][1] * il2;
+            b[v][kQuad0 + 2] = hb[F + v][2] * il2;
+            b[v][kQuad0 + 3] = 2.0 * hb[F + v][3] * il2;
+            b[v][kQuad0 + 4] = hb[F + v][4] * il2;
+            b[v][kQuad0 + 5] = 2.0 * hb[F + v][5] * il2;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) b[v][kLin0 + k] = gb[F + v][k] * il;
+          }
+          solve_thread<G, kQuad0, 0>(my, b);
+#pragma unroll
+          for (int v = 0; v < G; ++v)
+#pragma unroll
+            for (int k = 0; k < kNB; ++k) bbar[(F + v) * kNB + k] = b[v][k];
+        };
+        seeds(Num<0>{}, Num<4>{});
+        seeds(Num<4>{}, Num<3>{});
+      }
+      // mbar = fold of -sum_f bbar_f c_f^T onto the moments; the factor is dead
+      double mb[kNM];
+#pragma unroll
+      for (int k = 0; k < kNM; ++k) mb[k] = 0.0;
+#pragma unroll 1
+      for (int f = 0; f < kNFit; ++f) {
+        double bb[kNB], cc[kNB];
+#pragma unroll
+        for (int k = 0; k < kNB; ++k) {
+          bb[k] = bbar[f * kNB + k];
+          cc[k] = c[f * kNB + k];
+          my[(f * kNB + k) * 32] = bb[k];
+        }
+        mls_accum_mbar(bb, cc, mb);
+      }
+#pragma unroll
+      for (int k = 0; k < kNM; ++k) my[(kSlotMbar + k) * 32] = mb[k];
+    }
+    // backward pass over the neighbours: an entry's terms to its row, their
+    // negatives to particle i's own
+    const double xs = a.spos[s], ys = a.spos[N + s], zs = a.spos[2 * N + s];
+    const double dwd = a.weight_kind == 1 ? 0.0 : -4.0 * inv_rf2;
+    const volatile double* seed = my;  // read again for each neighbour rather than kept
+    const struct {
+      const volatile double* p;
+      __device__ __forceinline__ double operator[](int k) const { return p[k * 32]; }
+    } mbar{my + kSlotMbar * 32};
+    const int32_t* list = a.idx + beg;
+    double2* row = reinterpret_cast<double2*>(a.terms + (beg - row0) * kTerms);
+    const int longest = __reduce_max_sync(0xffffffffu, len);
+    int t = len > 0 ? list[0] : s;
+    double nx = a.spos[t], ny = a.spos[N + t], nz = a.spos[2 * N + t], nu[kNFit];
+#pragma unroll
+    for (int f = 0; f < kNFit; ++f) nu[f] = a.sU[(f + 1) * N + t];
+    t = len > 1 ? list[1] : s;
+#pragma unroll 1
+    for (int e = 0; e < longest; ++e) {
+      const double dx = wrap64(bx, 0, nx - xs), dy = wrap64(bx, 1, ny - ys), dz = wrap64(bx, 2, nz - zs);
+      double du[kNFit];
+#pragma unroll
+      for (int f = 0; f < kNFit; ++f) du[f] = nu[f] - u[f + 1];
+      // the next neighbour's values, a neighbour ahead
+      nx = a.spos[t];
+      ny = a.spos[N + t];
+      nz = a.spos[2 * N + t];
+#pragma unroll
+      for (int f = 0; f < kNFit; ++f) nu[f] = a.sU[(f + 1) * N + t];
+      t = e + 2 < len ? list[e + 2] : s;
+      bool inside;
+      const double s2 = dist_rel(dx, dy, dz, inv_rf2, inside);
+      if (e < len) {
+        double ub[kNFit], xb[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+        for (int f = 0; f < kNFit; ++f) ub[f] = 0.0;
+        if (inside && live) {
+          const double sw = 1.0 - s2;
+          const double wt = a.weight_kind == 1 ? 1.0 : sw * sw;
+          const double x = dx * il, y = dy * il, z = dz * il;
+          double p[kNB], Bt[kNB];
+          mls_basis(x, y, z, p);
+#pragma unroll
+          for (int k = 0; k < kNB; ++k) Bt[k] = 0.0;
+#pragma unroll
+          for (int f = 0; f < kNFit; ++f) {
+            double pb = 0.0;
+#pragma unroll
+            for (int k = 0; k < kNB; ++k) {
+              const double bk = seed[(f * kNB + k) * 32];
+              pb = fma(p[k], bk, pb);
+              Bt[k] = fma(du[f], bk, Bt[k]);
+            }
+            ub[f] = wt * pb;
+            selfu[f + 1] -= ub[f];
+          }
+          double P, Px, Py, Pz;
+          mls_poly_grad(x, y, z, mbar, Bt, P, Px, Py, Pz);
+          const double dw = P * dwd * sw;  // d w / d d = -4 (1 - s^2) d / r_f^2
+          const double wl = wt * il;
+          xb[0] = fma(wl, Px, dw * dx);
+          xb[1] = fma(wl, Py, dw * dy);
+          xb[2] = fma(wl, Pz, dw * dz);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) selfx[k] -= xb[k];
+        }
+        double2* to = row + e * (kTerms / 2);
+        to[0] = make_double2(ub[0], ub[1]);
+        to[1] = make_double2(ub[2], ub[3]);
+        to[2] = make_double2(ub[4], ub[5]);
+        to[3] = make_double2(ub[6], xb[0]);
+        to[4] = make_double2(xb[1], xb[2]);
+      }
+      __syncwarp();
+    }
+    if (act) {
+      for (int k = 0; k < 8; ++k) a.acc[k * N + s] += selfu[k];
+      for (int k = 0; k < 3; ++k) a.acc[(8 + k) * N + s] += selfx[k];
+    }
+    __syncwarp();
   }
 }
 
-// Own terms plus the contribution of every particle i whose list names t,
-// recomputed from i's seeds in ascending order of i; caller order out.
-__global__ void __launch_bounds__(128) k_adj_gather(const AdjArgs a, const int64_t* __restrict__ roff,
-                                                    const int32_t* __restrict__ rsrc,
+// ---- reverse neighbour lists of a chunk: for every particle t, the chunk's
+// entries that name t (numbered from the chunk's first).  A thread per entry.
+template <bool FILL>
+__global__ void __launch_bounds__(kThreads) k_rev(const __grid_constant__ AdjArgs a, int32_t* __restrict__ rcnt,
+                                                  const int64_t* __restrict__ roff,
+                                                  uint32_t* __restrict__ rsrc) {
+  int first, last;
+  chunk_slots(a, first, last);
+  if (first >= last) return;
+  const int64_t e0 = a.off[first];
+  const int64_t e1 = a.off[last] < a.g.capacity ? a.off[last] : a.g.capacity;
+  for (int64_t e = e0 + static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; e < e1;
+       e += static_cast<int64_t>(gridDim.x) * kThreads) {
+    const int t = a.idx[e];
+    const int k = atomicAdd(&rcnt[t], 1);
+    if (FILL) rsrc[roff[t] + k] = static_cast<uint32_t>(e - e0);
+  }
+}
+
+// Add the chunk's rows that name t to t's sums: a warp per particle.  The
+// atomics left its entries in any order: each entry's rank among them (their
+// number smaller than it) puts them in order in shared memory, 32 at a time,
+// then three groups of ten lanes sum every third row, a column per lane, so
+// that a row is read as one piece.  With the last chunk the sums go out in
+// caller order.
+__global__ void __launch_bounds__(128) k_adj_gather(const __grid_constant__ AdjArgs a,
+                                                    const int64_t* __restrict__ roff,
+                                                    const uint32_t* __restrict__ rsrc,
                                                     double* __restrict__ Ubar,
                                                     double* __restrict__ xbar) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= a.n) return;
+  constexpr int kRegs = 4;  // entries per lane kept in registers; longer lists are read again
+  __shared__ uint32_t sorted[4][32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t w = static_cast<int64_t>(blockIdx.x) * 4 + wid;
+  if (w >= a.n) return;
+  const int t = static_cast<int>(w);
   const int64_t N = a.n;
-  double len[3], ilen[3];
-  for (int c = 0; c < 3; ++c) {
-    len[c] = a.g.len[c];
-    ilen[c] = a.g.periodic[c] ? 1.0 / a.g.len[c] : 0.0;
+  const int64_t r0 = roff[t];
+  const int m = static_cast<int>(roff[t + 1] - r0);
+  uint32_t v[kRegs];
+  int rank[kRegs];
+#pragma unroll
+  for (int q = 0; q < kRegs; ++q) {
+    v[q] = q * 32 + lane < m ? rsrc[r0 + q * 32 + lane] : 0xffffffffu;
+    rank[q] = 0;
   }
-  double acc[11];
-  for (int k = 0; k < 11; ++k) acc[k] = a.self[k * N + t];
-  for (int64_t r = roff[t]; r < roff[t + 1]; ++r) {
-    const int i = rsrc[r];
-    double u[8];
-    for (int f = 0; f < 8; ++f) u[f] = a.sU[f * N + i];
-    const double lam = a.slam[i];
-    const double rf = a.g.rf_factor * lam;
-    const double* bb = a.scr + static_cast<int64_t>(i) * kScr;
-    double ub[kNFit], xb[3];
-    if (!entry_adjoint(a, t, a.spos[i], a.spos[N + i], a.spos[2 * N + i], u, 1.0 / (rf * rf),
-                       1.0 / lam, len, ilen, bb + kScrBbar, 1, bb + kScrMbar, 1, ub, xb))
-      continue;
-    for (int k = 0; k < kNFit; ++k) acc[1 + k] += ub[k];
-    for (int c = 0; c < 3; ++c) acc[8 + c] += xb[c];
+  const int near = m < 32 * kRegs ? m : 32 * kRegs;
+#pragma unroll
+  for (int q = 0; q < kRegs; ++q)
+    for (int j = 0; j < 32 && q * 32 + j < near; ++j) {
+      const uint32_t x = __shfl_sync(0xffffffffu, v[q], j);
+#pragma unroll
+      for (int k = 0; k < kRegs; ++k) rank[k] += x < v[k] ? 1 : 0;
+    }
+  for (int j = near; j < m; ++j) {
+    const uint32_t x = rsrc[r0 + j];
+#pragma unroll
+    for (int k = 0; k < kRegs; ++k) rank[k] += x < v[k] ? 1 : 0;
+  }
+  const int grp = lane / kTerms, col = lane - grp * kTerms;
+  double acc = 0.0;
+  for (int base = 0; base < m; base += 32) {
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < kRegs; ++q)
+      if (q * 32 + lane < m && rank[q] >= base && rank[q] < base + 32) sorted[wid][rank[q] - base] = v[q];
+    for (int j = near + lane; j < m; j += 32) {  // entries beyond the registers
+      const uint32_t x = rsrc[r0 + j];
+      int r = 0;
+      for (int i = 0; i < m; ++i) r += rsrc[r0 + i] < x ? 1 : 0;
+      if (r >= base && r < base + 32) sorted[wid][r - base] = x;
+    }
+    __syncwarp();
+    const int cnt = m - base < 32 ? m - base : 32;
+    if (grp < 3)
+#pragma unroll 4
+      for (int j = grp; j < cnt; j += 3) acc += a.terms[static_cast<int64_t>(sorted[wid][j]) * kTerms + col];
+  }
+  const double s1 = __shfl_down_sync(0xffffffffu, acc, kTerms);
+  const double s2 = __shfl_down_sync(0xffffffffu, acc, 2 * kTerms);
+  acc += s1 + s2;
+  // columns 0..6: Ubar of fields 1..7, 7..9: xbar; Ubar of field 0 has own terms only
+  const bool done = a.chunk == a.chunks - 1;
+  const int k = lane < kTerms ? lane + 1 : 0;
+  if (lane > kTerms) return;
+  double* sum = a.acc + k * N + t;
+  const double total = lane < kTerms ? *sum + acc : *sum;
+  if (!done) {
+    *sum = total;
+    return;
   }
   const int i = a.perm[t];
-  for (int k = 0; k < 8; ++k) Ubar[k * N + i] = acc[k];
-  for (int c = 0; c < 3; ++c) xbar[c * N + i] = acc[8 + c];
+  if (k < 8) Ubar[k * N + i] = total;
+  else xbar[(k - 8) * N + i] = total;
 }
 
 }  // namespace
@@ -521,6 +558,7 @@ phb_status adjoint_impl(int mode, const phb_plan* plan, const phb_params* prm, c
   a.g = g;
   a.n = n;
   a.perm = region<int32_t>(plan, ws, R_PERM);
+  a.tmap = region<uint8_t>(plan, ws, R_TMAP);
   a.spos = region<double>(plan, ws, R_SPOS);
   a.slam = region<double>(plan, ws, R_SLAM);
   a.sU = region<double>(plan, ws, R_SU);
@@ -534,45 +572,43 @@ phb_status adjoint_impl(int mode, const phb_plan* plan, const phb_params* prm, c
   a.c_zeta_l = prm->c_zeta_l;
   a.c_zeta_a = prm->c_zeta_a;
   a.c_eta = prm->c_eta;
-  a.scr = region<double>(plan, ws, R_ADJ_SCR);
-  a.self = region<double>(plan, ws, R_ADJ_SELF);
+  a.terms = region<double>(plan, ws, R_ADJ_TERMS);
+  a.acc = region<double>(plan, ws, R_ADJ_ACC);
   a.rec = rec;
   a.status_word = status_word;
-  const size_t smem = size_t(kSm) * kT * sizeof(double);
-  const unsigned grid = static_cast<unsigned>((n + kT - 1) / kT);
-  if (mode == kRecompute) {
-    cudaFuncSetAttribute(k_adjoint<kRecompute>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(smem));
-    k_adjoint<kRecompute><<<grid, kT, smem, st>>>(a);
-  } else if (mode == kRecord) {
-    cudaFuncSetAttribute(k_adjoint<kRecord>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(smem));
-    k_adjoint<kRecord><<<grid, kT, smem, st>>>(a);
+  a.span = adjoint_rows(plan) - n;
+  a.chunk = 0;
+  a.chunks = static_cast<int32_t>(plan->nbr_capacity > a.span ? (plan->nbr_capacity + a.span - 1) / a.span : 1);
+  const size_t smem = size_t(kSlots) * kT * sizeof(double);
+  const unsigned grid = static_cast<unsigned>(num_sms());
+  const auto kernel = mode == kRecompute ? k_adjoint<kRecompute>
+                      : mode == kRecord  ? k_adjoint<kRecord>
+                                         : k_adjoint<kStored>;
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (mode == kRecord) {
+    kernel<<<grid, kT, smem, st>>>(a);
     note_launch();
     return launch_status(cudaSuccess);
-  } else {
-    cudaFuncSetAttribute(k_adjoint<kStored>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(smem));
-    k_adjoint<kStored><<<grid, kT, smem, st>>>(a);
   }
-  note_launch();
   int32_t* rcnt = region<int32_t>(plan, ws, R_ADJ_RCNT);
   int64_t* roff = region<int64_t>(plan, ws, R_ADJ_ROFF);
-  int32_t* rsrc = region<int32_t>(plan, ws, R_ADJ_RSRC);
+  uint32_t* rsrc = region<uint32_t>(plan, ws, R_ADJ_RSRC);
   int64_t* bsum = region<int64_t>(plan, ws, R_SCAN);
-  const int64_t cap = plan->nbr_capacity;
-  const unsigned nb = static_cast<unsigned>((n + kThreads - 1) / kThreads);
-  if ((e = cudaMemsetAsync(rcnt, 0, (n + 1) * sizeof(int32_t), st))) return launch_status(e);
-  k_rev_count<<<nb, kThreads, 0, st>>>(n, cap, a.off, a.idx, rcnt);
-  note_launch();
-  if ((e = scan_exclusive_i32_to_i64(rcnt, roff, n + 1, bsum, st))) return launch_status(e);
-  if ((e = cudaMemsetAsync(rcnt, 0, (n + 1) * sizeof(int32_t), st))) return launch_status(e);
-  k_rev_fill<<<nb, kThreads, 0, st>>>(n, cap, a.off, a.idx, roff, rcnt, rsrc);
-  note_launch();
-  k_rev_sort<<<nb, kThreads, 0, st>>>(n, roff, rsrc);
-  note_launch();
-  k_adj_gather<<<static_cast<unsigned>((n + 127) / 128), 128, 0, st>>>(a, roff, rsrc, Ubar, xbar);
-  note_launch();
+  const size_t cnt_bytes = (size_t(n) + 1) * sizeof(int32_t);
+  if ((e = cudaMemsetAsync(a.acc, 0, size_t(11) * n * sizeof(double), st))) return launch_status(e);
+  for (a.chunk = 0; a.chunk < a.chunks; ++a.chunk) {
+    if ((e = cudaMemsetAsync(rcnt, 0, cnt_bytes, st))) return launch_status(e);
+    k_rev<false><<<grid * 8, kThreads, 0, st>>>(a, rcnt, nullptr, nullptr);
+    note_launch();
+    if ((e = scan_exclusive_i32_to_i64(rcnt, roff, n + 1, bsum, st))) return launch_status(e);
+    if ((e = cudaMemsetAsync(rcnt, 0, cnt_bytes, st))) return launch_status(e);
+    k_rev<true><<<grid * 8, kThreads, 0, st>>>(a, rcnt, roff, rsrc);
+    note_launch();
+    kernel<<<grid, kT, smem, st>>>(a);
+    note_launch();
+    k_adj_gather<<<static_cast<unsigned>((n + 3) / 4), 128, 0, st>>>(a, roff, rsrc, Ubar, xbar);
+    note_launch();
+  }
   return launch_status(cudaSuccess);
 }
 

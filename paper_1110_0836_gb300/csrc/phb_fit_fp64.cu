@@ -29,8 +29,7 @@
 // r_j = (U_j - U_i) - p(q_j).c are recomputed from the data, A^T W r is
 // accumulated again and solved with the same factor, so the error follows
 // cond(A) rather than cond(A^T W A) = cond(A)^2.
-#include "phb_internal.cuh"
-#include "mls_gen.cuh"
+#include "phb_fit64.cuh"
 #include "phb_mhd.cuh"
 
 namespace phb {
@@ -40,10 +39,7 @@ constexpr int kWarps = 4;  // per block, one block per SM: one warp per sub-part
 constexpr int kT = 32 * kWarps;
 
 // Thread form: a warp's shared memory is [slot][32 lanes] doubles.
-constexpr int kSlots = kNT;              // the factor: 190 doubles per thread, 190 KB per block
-constexpr int kSlotOwn = kNF * kNB;      // while accumulating: x, y, z, 1/lambda, 1/r_f^2, U
-constexpr int kSlotNbr = kSlotOwn + 13;  // and two neighbours' x, y, z, U, the next one on its way
-static_assert(kSlotNbr + 2 * 11 <= kNT, "accumulators and own values must fit below the factor's end");
+constexpr int kSlots = kNT;  // the factor: 190 doubles per thread, 190 KB per block
 
 // Warp form: per warp, doubles.
 constexpr int kRow = 39;                 // staged neighbour: w, w q^cubic (10), w dU (8), q^basis (19); odd stride
@@ -54,102 +50,6 @@ constexpr int kWM = kWC + kNF * kNB;     // moments
 constexpr int kWI = kWM + kNM;           // 1 / L_kk
 constexpr int kWarpSlots = kWI + kNB;
 static_assert(kWarpSlots <= kSlots * 32, "the warp form runs in the thread form's shared memory");
-
-__device__ __forceinline__ int tri0(int r) { return r * (r + 1) / 2; }
-
-struct Box64 {
-  double len[3], inv_len[3];
-  int far[3];  // high word of a quarter box length: below it an offset is its minimum image
-};
-
-__device__ __forceinline__ Box64 make_box64(const Grid& g) {
-  Box64 b;
-  for (int c = 0; c < 3; ++c) {
-    b.len[c] = g.len[c];
-    b.inv_len[c] = g.periodic[c] ? 1.0 / g.len[c] : 0.0;
-    b.far[c] = g.periodic[c] ? __double2hiint(0.25 * g.len[c]) : 0x7fffffff;
-  }
-  return b;
-}
-
-// d - len rint(d / len) (the wrap only where it changes something)
-__device__ __forceinline__ double wrap64(const Box64& b, int c, double d) {
-  if ((__double2hiint(d) & 0x7fffffff) >= b.far[c]) d = fma(-b.len[c], rint(d * b.inv_len[c]), d);
-  return d;
-}
-
-// Squared distance over r_f^2; `inside` (s2 < 1) from the exponent bits: s2 >= 0
-// or NaN, whose high word lies above that of 1.
-__device__ __forceinline__ double dist_rel(double dx, double dy, double dz, double inv_rf2, bool& inside) {
-  const double s2 = fma(dz, dz, fma(dy, dy, __dmul_rn(dx, dx))) * inv_rf2;
-  inside = __double2hiint(s2) < 0x3ff00000;
-  return s2;
-}
-
-__device__ __forceinline__ double weight64(double s2, int weight_kind) {
-  const double sw = __dadd_rn(1.0, -s2);
-  return weight_kind == 1 ? 1.0 : __dmul_rn(sw, sw);
-}
-
-// v truncated to FP32 on the integer pipe (for the conditioning estimate).
-__device__ __forceinline__ float f32_of(double v) {
-  const unsigned hi = static_cast<unsigned>(__double2hiint(v));
-  const unsigned mag = hi & 0x7fffffffu;
-  unsigned r = __funnelshift_l(static_cast<unsigned>(__double2loint(v)), mag - 0x38000000u, 3);
-  r = mag < 0x38100000u ? 0u : (mag >= 0x47f00000u ? 0x7f7fffffu : r);
-  return __uint_as_float(r | (hi & 0x80000000u));
-}
-
-template <int N>
-struct Num {
-  static constexpr int value = N;
-};
-
-// Cholesky of columns C0 .. C0 + W - 1 of the factor in a thread's column (my,
-// stride 32), the columns before them done: the panel in registers, so that
-// its independent FMAs cover the shared-memory loads (loops of dot products
-// through shared memory took 290 cycles per FMA, this form ~90).  The diagonal
-// slots take 1 / L_kk, mkk the diagonal of M in FP32.  A Jacobi-scaled pivot
-// below 1e-12 (cond(M) above ~1e12) is treated as singular.
-template <int C0, int W>
-__device__ __forceinline__ void chol_panel(double* my, float (&mkk)[kNB], bool& singular) {
-  constexpr int R = kNB - C0;
-  double v[W][R];
-  double d[W];
-#pragma unroll
-  for (int c = 0; c < W; ++c) {
-#pragma unroll
-    for (int r = c; r < R; ++r) v[c][r] = my[(tri0(C0 + r) + C0 + c) * 32];
-    d[c] = v[c][c];
-    mkk[C0 + c] = f32_of(d[c]);
-  }
-#pragma unroll 1
-  for (int k = 0; k < C0; ++k) {
-    double l[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) l[r] = my[(tri0(C0 + r) + k) * 32];
-#pragma unroll
-    for (int c = 0; c < W; ++c)
-#pragma unroll
-      for (int r = c; r < R; ++r) v[c][r] = fma(-l[r], l[c], v[c][r]);
-  }
-#pragma unroll
-  for (int c = 0; c < W; ++c) {
-    const double p = v[c][c];
-    singular |= !(p > 0.0) || !(p > 1e-12 * d[c]);
-    const double inv = rsqrt(p > 0.0 ? p : 1.0);
-    my[(tri0(C0 + c) + C0 + c) * 32] = inv;
-#pragma unroll
-    for (int r = c + 1; r < R; ++r) {
-      v[c][r] *= inv;
-      my[(tri0(C0 + r) + C0 + c) * 32] = v[c][r];
-    }
-#pragma unroll
-    for (int e = c + 1; e < W; ++e)
-#pragma unroll
-      for (int r = e; r < R; ++r) v[e][r] = fma(-v[c][r], v[c][e], v[e][r]);
-  }
-}
 
 // Estimate of ||M_s^-1||_inf of the Jacobi-scaled matrix (as mls_inv_norm_est,
 // the back substitution by columns) in FP32 from the factor in a thread's
@@ -177,49 +77,6 @@ __device__ __forceinline__ float inv_norm_est(const double* my, const float (&mk
     for (int i = 0; i < k; ++i) y[i] = fmaf(-f32_of(L[(tri0(k) + i) * 32]), y[k], y[i]);
   }
   return mx;
-}
-
-// Substitutions of NF right-hand sides at once in registers, with the factor
-// in a thread's column: coefficients kQuad0 .. 18 (linear and quadratic).
-template <int NF>
-__device__ __forceinline__ void solve_thread(const double* factor, double (&b)[NF][kNB]) {
-  const volatile double* my = factor;  // read again by each group of fields rather than kept
-#pragma unroll
-  for (int i = 0; i < kNB; ++i) {
-#pragma unroll
-    for (int k = 0; k < i; ++k) {
-      const double l = my[(tri0(i) + k) * 32];
-#pragma unroll
-      for (int f = 0; f < NF; ++f) b[f][i] = fma(-l, b[f][k], b[f][i]);
-    }
-    const double inv = my[(tri0(i) + i) * 32];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) b[f][i] *= inv;
-  }
-#pragma unroll
-  for (int i = kNB - 1; i >= kQuad0; --i) {
-#pragma unroll
-    for (int k = kNB - 1; k > i; --k) {
-      const double l = my[(tri0(k) + i) * 32];
-#pragma unroll
-      for (int f = 0; f < NF; ++f) b[f][i] = fma(-l, b[f][k], b[f][i]);
-    }
-    const double inv = my[(tri0(i) + i) * 32];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) b[f][i] *= inv;
-  }
-}
-
-// Gradient and packed Hessian from a field's linear and quadratic coefficients.
-template <class C>
-__device__ __forceinline__ void derivs_of(C c, double il, double il2, double (&g)[3], double (&h)[6]) {
-  for (int k = 0; k < 3; ++k) g[k] = c(kLin0 + k) * il;
-  h[0] = 2.0 * c(kQuad0) * il2;
-  h[1] = c(kQuad0 + 1) * il2;
-  h[2] = c(kQuad0 + 2) * il2;
-  h[3] = 2.0 * c(kQuad0 + 3) * il2;
-  h[4] = c(kQuad0 + 4) * il2;
-  h[5] = 2.0 * c(kQuad0 + 5) * il2;
 }
 
 __device__ __forceinline__ void write_derivs(const FitArgs& a, int f, int dst, const double (&g)[3],
@@ -250,16 +107,9 @@ __device__ __noinline__ void write_rhs(const FitArgs& a, int s, int dst, const M
   if (!finite) raise_flag(a.status_word, PHB_FLAG_NONFINITE);
 }
 
-__device__ __forceinline__ int64_t list_end(const FitArgs& a, int s) {
-  const int64_t e = a.off[s + 1];
-  return e < a.g.capacity ? e : a.g.capacity;
-}
-
 // One particle per lane (slot < 0: none); my: the lane's shared-memory column
-// (stride 32).  All lanes call it, and the lanes meet again after every
-// neighbour: left to themselves the lanes of lists of different lengths ran
-// the loop apart, in up to twice the time.  Returns true, with nothing
-// written, when the fit needs the corrected step.
+// (stride 32).  All lanes call it.  Returns true, with nothing written, when
+// the fit needs the corrected step.
 template <FitMode MODE>
 __device__ __forceinline__ bool fit_thread(const FitArgs& a, const Box64& bx, int slot, bool routed,
                                            float refine_above, double* my) {
@@ -268,79 +118,12 @@ __device__ __forceinline__ bool fit_thread(const FitArgs& a, const Box64& bx, in
   const int s = slot < 0 ? 0 : slot;
   const double lam = a.slam[s];
   const double inv_l = 1.0 / lam;
+  const double rf = a.g.rf_factor * lam;
   const int64_t beg = a.off[s];
-  const int len = slot < 0 ? 0 : static_cast<int>(list_end(a, s) - beg);
-  const int longest = __reduce_max_sync(0xffffffffu, len);
-  // the particle's own values in shared memory, read when used: registers
-  // hold the 80 moments
-  volatile double* own = my + kSlotOwn * 32;
-  {
-    const double rf = a.g.rf_factor * lam;
-    for (int c = 0; c < 3; ++c) own[c * 32] = a.spos[c * n + s];
-    own[3 * 32] = inv_l;
-    own[4 * 32] = 1.0 / (rf * rf);
-    for (int f = f0; f < kNF; ++f) own[(5 + f) * 32] = a.sU[f * n + s];
-  }
-  for (int k = f0 * kNB; k < kNF * kNB; ++k) my[k * 32] = 0.0;
+  const int len = slot < 0 ? 0 : list_len64(a.off, a.g.capacity, s);
   double m[kNM];
-#pragma unroll
-  for (int k = 0; k < kNM; ++k) m[k] = 0.0;
-  int cnt = 0;
-  // the next neighbour's values are copied to shared memory during this one's
-  // sums (no registers, and their latency, ~1,400 cycles a neighbour, hidden)
-  constexpr int kNbr = 3 + kNF - f0;
-  volatile double* nbr = my + kSlotNbr * 32;
-  auto fetch = [&](int t, int e) {
-    const unsigned to = static_cast<unsigned>(__cvta_generic_to_shared(my + (kSlotNbr + (e & 1) * kNbr) * 32));
-#pragma unroll
-    for (int c = 0; c < kNbr; ++c) {
-      const double* from = c < 3 ? a.spos + c * n + t : a.sU + (f0 + c - 3) * n + t;
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(to + c * 256), "l"(from) : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  const int32_t* list = a.idx + beg;
-  fetch(len > 0 ? list[0] : s, 0);
-  int next = len > 1 ? list[1] : s;
-#pragma unroll 1
-  for (int e = 0; e < longest; ++e) {
-    fetch(next, e + 1);
-    next = e + 2 < len ? list[e + 2] : s;
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    const volatile double* at = nbr + (e & 1) * kNbr * 32;
-    const double dx = wrap64(bx, 0, at[0] - own[0]);
-    const double dy = wrap64(bx, 1, at[32] - own[32]);
-    const double dz = wrap64(bx, 2, at[64] - own[64]);
-    bool inside;
-    const double s2 = dist_rel(dx, dy, dz, own[4 * 32], inside);
-    if (inside && e < len) {
-      ++cnt;
-      const double wt = weight64(s2, a.weight_kind);
-      double qg[kNB], wq[kNB + 1];
-      const double il = own[3 * 32];
-      mls_monomials_cubic_w(dx * il, dy * il, dz * il, wt, qg, wq);
-      // the sums in shared memory are loaded two ahead: with the moments in
-      // registers the compiler otherwise loads each just before its FMA
-      // (123 instead of 70 cycles per FMA)
-      volatile double* b = my + f0 * kNB * 32;
-      constexpr int N = (kNF - f0) * kNB;
-      double ahead[2] = {b[0], b[32]};
-#pragma unroll
-      for (int f = f0; f < kNF; ++f) {
-        const double wdu = wt * (at[(3 + f - f0) * 32] - own[(5 + f) * 32]);
-#pragma unroll
-        for (int k = 0; k < kNB; ++k) {
-          const int i = (f - f0) * kNB + k;
-          const double v = ahead[i & 1];
-          if (i + 2 < N) ahead[i & 1] = b[(i + 2) * 32];
-          b[i * 32] = fma(qg[k], wdu, v);
-        }
-      }
-      mls_accum_moments(qg, wq, m);
-    }
-    __syncwarp();
-  }
-  asm volatile("cp.async.wait_all;" ::: "memory");
+  const int cnt = accum_thread<f0>(a.spos, a.sU, n, a.idx + beg, len, s, bx, a.weight_kind, inv_l,
+                                   1.0 / (rf * rf), my, m);
   // the right-hand sides to local memory, the normal matrix in their place
   double b[kNF * kNB];
 #pragma unroll 4
@@ -375,7 +158,7 @@ __device__ __forceinline__ bool fit_thread(const FitArgs& a, const Box64& bx, in
     for (int u = 0; u < N; ++u)
 #pragma unroll
       for (int k = 0; k < kNB; ++k) c[u][k] = b[(f + u) * kNB + k];
-    solve_thread(my, c);
+    solve_thread<N, 0, kQuad0>(my, c);
 #pragma unroll
     for (int u = 0; u < N; ++u) {
       double g[3] = {0, 0, 0}, h[6] = {0, 0, 0, 0, 0, 0};
@@ -440,7 +223,7 @@ __device__ __forceinline__ int warp_sums(const FitArgs& a, const Box64& bx, cons
   constexpr int nsum = kNM + (kNF - f0) * kNB;
   constexpr int rounds = (nsum + 31) / 32;
   const int64_t n = a.n;
-  const int64_t beg = a.off[s], end = list_end(a, s);
+  const int64_t beg = a.off[s], end = beg + list_len64(a.off, a.g.capacity, s);
   const double xs = a.spos[s], ys = a.spos[n + s], zs = a.spos[2 * n + s];
   double acc[rounds];
 #pragma unroll

@@ -59,10 +59,10 @@ enum Region {
   R_PC_IO,       // double [12][n] pos, lambda, U (caller order) of phb_pc_step_host -- PC step
   R_PC_DONE,     // uint8 [n] slots whose U^{n+1} the corrector's fit wrote to the host -- PC step
   R_ADJ_ROFF,    // int64 [n+1] reverse-list offsets                     -- adjoint
-  R_ADJ_RSRC,    // int32 [capacity] reverse lists: the particles naming each particle -- adjoint
+  R_ADJ_RSRC,    // uint32 [rows] reverse lists: the chunk's entries naming each particle -- adjoint
   R_ADJ_RCNT,    // int32 [n+1] reverse-list counts / cursors            -- adjoint
-  R_ADJ_SCR,     // double [n][266] per particle: seeds bbar, coefficients c then mbar -- adjoint
-  R_ADJ_SELF,    // double [11][n] each particle's own adjoint terms      -- adjoint
+  R_ADJ_TERMS,   // double [rows][10] adjoint terms of a chunk's list entries -- adjoint
+  R_ADJ_ACC,     // double [11][n] Ubar and xbar so far (slot order)      -- adjoint
   R_END_COMMON,  // end of the common part (prefix for RHS / derivs)
   R_END,         // end of everything
   R_END_PC,      // end of the PC-step regions
@@ -98,6 +98,13 @@ struct Grid {
 };
 
 Grid make_grid(const phb_plan* p);
+
+// Rows (list entries) of the adjoint's term buffer: all list entries of sets up
+// to 2^17 particles (2^23 rows at most), else 28 per particle - the entries
+// then go through it in chunks of rows - n (a list is shorter than n), two at
+// ~52 neighbours, in no more memory than a record of seeds and coefficients
+// per particle took.
+int64_t adjoint_rows(const phb_plan* p);
 
 __device__ __forceinline__ float phb_rsqrt(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double phb_rsqrt(double x) { return 1.0 / sqrt(x); }

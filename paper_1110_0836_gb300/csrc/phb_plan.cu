@@ -46,6 +46,11 @@ Grid make_grid(const phb_plan* p) {
   return g;
 }
 
+int64_t adjoint_rows(const phb_plan* p) {
+  const int64_t all = std::max<int64_t>(p->nbr_capacity, 1) + p->n, some = 28 * p->n;
+  return p->n > int64_t(1) << 17 ? some : std::max(some, std::min<int64_t>(all, int64_t(1) << 23));
+}
+
 int num_sms() {
   static int sms = 0;
   if (!sms) {
@@ -362,12 +367,12 @@ extern "C" phb_status phb_plan_init(phb_plan* p) {
   p->ws_off[R_ADJ_ROFF] = ad;
   ad += align256(size_t(n + 1) * 8);
   p->ws_off[R_ADJ_RSRC] = ad;
-  ad += align256(size_t(cap) * 4);
+  ad += align256(size_t(adjoint_rows(p)) * 4);
   p->ws_off[R_ADJ_RCNT] = ad;
   ad += align256(size_t(n + 1) * 4);
-  p->ws_off[R_ADJ_SCR] = ad;
-  ad += align256(size_t(266) * n * 8);
-  p->ws_off[R_ADJ_SELF] = ad;
+  p->ws_off[R_ADJ_TERMS] = ad;
+  ad += align256(size_t(adjoint_rows(p)) * 80);
+  p->ws_off[R_ADJ_ACC] = ad;
   ad += align256(size_t(11) * n * 8);
   p->ws_off[R_END_PC] = pc;
   p->ws_off[R_END_ADJ] = ad;
