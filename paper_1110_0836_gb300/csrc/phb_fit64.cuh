@@ -41,10 +41,10 @@ __device__ __forceinline__ double wrap64(const Box64& b, int c, double d) {
 }
 
 // Squared distance over r_f^2; `inside` (s2 < 1) from the exponent bits: s2 >= 0
-// or NaN, whose high word lies above that of 1.
+// or a NaN of either sign, whose high word lies above that of 1.
 __device__ __forceinline__ double dist_rel(double dx, double dy, double dz, double inv_rf2, bool& inside) {
   const double s2 = fma(dz, dz, fma(dy, dy, __dmul_rn(dx, dx))) * inv_rf2;
-  inside = __double2hiint(s2) < 0x3ff00000;
+  inside = static_cast<unsigned>(__double2hiint(s2)) < 0x3ff00000u;
   return s2;
 }
 

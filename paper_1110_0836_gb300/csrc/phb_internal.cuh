@@ -172,9 +172,11 @@ static __device__ __noinline__ int cell_wrap_fp64(const Grid& g, int a, double t
       c -= nc;
       k += 1;
     }
+    // beyond 2^53 cells the remainder is lost to rounding: any cell will do
+    // (no sum over images is meant there), but it has to be one of the grid's
     k_out = k;
-    k_zero = false;
-    return static_cast<int>(c);
+    k_zero = !(c >= 0.0 && c < nc);
+    return k_zero ? 0 : static_cast<int>(c);
   }
   k_out = 0.0;
   k_zero = true;
