@@ -120,6 +120,21 @@ __device__ __forceinline__ bool finite64(double x) {
   return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
 }
 
+// v truncated to FP32 on the integer pipe.
+__device__ __forceinline__ float f32_of(double v) {
+  const unsigned hi = static_cast<unsigned>(__double2hiint(v));
+  const unsigned mag = hi & 0x7fffffffu;
+  unsigned r = __funnelshift_l(static_cast<unsigned>(__double2loint(v)), mag - 0x38000000u, 3);
+  r = mag < 0x38100000u ? 0u : (mag >= 0x47f00000u ? 0x7f7fffffu : r);
+  return __uint_as_float(r | (hi & 0x80000000u));
+}
+
+// Entries of slot s's list (those beyond the capacity were dropped).
+__device__ __forceinline__ int list_len64(const int64_t* off, int64_t capacity, int s) {
+  const int64_t b = off[s], e = off[s + 1] < capacity ? off[s + 1] : capacity;
+  return e > b ? static_cast<int>(e - b) : 0;
+}
+
 // Cell coordinate on one axis and the matching wrap count k: with
 // u = floor((x - lo) / cell) (reciprocal cell edge), a periodic axis gives
 // c = u - k nc, k = floor(u / nc), and the wrapped position x - k len lies in

@@ -919,15 +919,35 @@ __global__ void k_adapt_gather(Grid g, const int32_t* __restrict__ perm, const d
   scr[s] = make_float4(w[0], w[1], w[2], 0.f);
 }
 
-constexpr int kGrid = 9;                       // test points per axis
-constexpr int kGridPts = kGrid * kGrid * kGrid;
+// Grid points k (9 per axis, index ((kx+4) 9 + (ky+4)) 9 + (kz+4)) with
+// |k|^2 <= Q2, in ascending index.
+template <int Q2>
+struct GridPoints {
+  int n = 0;
+  int8_t x[257] = {}, y[257] = {}, z[257] = {};
+  constexpr GridPoints() {
+    for (int i = -4; i <= 4; ++i)
+      for (int j = -4; j <= 4; ++j)
+        for (int k = -4; k <= 4; ++k)
+          if (i * i + j * j + k * k <= Q2) {
+            x[n] = static_cast<int8_t>(i);
+            y[n] = static_cast<int8_t>(j);
+            z[n] = static_cast<int8_t>(k);
+            ++n;
+          }
+  }
+};
+constexpr int grid_points(int q2) { return q2 == 5 ? 57 : 257; }
+static_assert(GridPoints<5>().n == grid_points(5) && GridPoints<16>().n == grid_points(16), "point counts");
+__device__ constexpr GridPoints<5> kGrid5;
+__device__ constexpr GridPoints<16> kGrid16;
 
 // FP32 offset of record o from me, minimum image on periodic axes.
-__device__ __forceinline__ float3 offset32(const Screen& q, float4 me, float4 o) {
+__device__ __forceinline__ float3 offset32(const Grid& g, float4 me, float4 o) {
   float dx = o.x - me.x, dy = o.y - me.y, dz = o.z - me.z;
-  dx = fmaf(-q.lenf[0], rintf(dx * q.invlf[0]), dx);
-  dy = fmaf(-q.lenf[1], rintf(dy * q.invlf[1]), dy);
-  dz = fmaf(-q.lenf[2], rintf(dz * q.invlf[2]), dz);
+  dx = fmaf(-g.lenf[0], rintf(dx * g.inv_lenf[0]), dx);
+  dy = fmaf(-g.lenf[1], rintf(dy * g.inv_lenf[1]), dy);
+  dz = fmaf(-g.lenf[2], rintf(dz * g.inv_lenf[2]), dz);
   return make_float3(dx, dy, dz);
 }
 
@@ -943,147 +963,251 @@ __device__ __forceinline__ double test_dist2(const Grid& g, const double* spos, 
   return __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
 }
 
-// Thread per slot.  Every FP64 quantity that decides an output is computed
-// with single IEEE-rounded operations in the order of the definition; FP32
-// screens with a margin only skip work whose outcome they prove.
-__global__ void __launch_bounds__(128) k_adapt_scan(Grid g, const int32_t* __restrict__ perm,
+// Exact squared distance from neighbour t of slot s to the test point (kx, ky,
+// kz), below d_v^2.
+__device__ __forceinline__ bool covers_exact(const Grid& g, const double* spos, int s, int t, double lam,
+                                          double vf, int kx, int ky, int kz) {
+  const double h = __dmul_rn(__dmul_rn(g.rf_factor, lam), 0.25), v = __dmul_rn(vf, lam);
+  return test_dist2(g, spos, g.n, s, t, __dmul_rn(static_cast<double>(kx), h),
+                    __dmul_rn(static_cast<double>(ky), h), __dmul_rn(static_cast<double>(kz), h)) <
+         __dmul_rn(v, v);
+}
+
+__device__ __forceinline__ bool closer_exact(const Grid& g, const double* spos, int s, int t, double lam,
+                                          double cf) {
+  const double c = __dmul_rn(cf, lam);
+  return dist2_exact(g, spos, g.n, s, t) < __dmul_rn(c, c);
+}
+
+// Exact clearance squared of test point (kx, ky, kz) of slot s (all lanes of a
+// warp): the smallest squared distance to the particle and its r_f set.  Only
+// entries within near2 (FP32) can hold it.
+__device__ __forceinline__ double clearance_exact(const Grid& g, const double* spos, const float4* scr,
+                                               const int32_t* idx, int64_t beg, int64_t end, int s,
+                                               double lam, int kx, int ky, int kz, float near2) {
+  const float4 me = scr[s];
+  const double rr = __dmul_rn(g.rf_factor, lam), h = __dmul_rn(rr, 0.25);
+  const double ox = __dmul_rn(static_cast<double>(kx), h), oy = __dmul_rn(static_cast<double>(ky), h),
+               oz = __dmul_rn(static_cast<double>(kz), h);
+  const float fx = __double2float_rn(ox), fy = __double2float_rn(oy), fz = __double2float_rn(oz);
+  double c = __dadd_rn(__dadd_rn(__dmul_rn(ox, ox), __dmul_rn(oy, oy)), __dmul_rn(oz, oz));
+  for (int64_t e = beg + (threadIdx.x & 31); e < end; e += 32) {
+    const int t = idx[e];
+    const float3 d = offset32(g, me, scr[t]);
+    const float ex = d.x - fx, ey = d.y - fy, ez = d.z - fz;
+    if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) > near2) continue;
+    if (!(dist2_exact(g, spos, g.n, s, t) < __dmul_rn(rr, rr))) continue;  // a skin entry, not in N(i)
+    const double e2 = test_dist2(g, spos, g.n, s, t, ox, oy, oz);
+    c = e2 < c ? e2 : c;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double x = __shfl_xor_sync(0xffffffffu, c, o);
+    c = x < c ? x : c;
+  }
+  return c;
+}
+
+// What the scan asks of every particle alike.
+struct ScanRule {
+  double vf, cf;
+  uint32_t test;  // bit q: points with |k|^2 = q are tested (neither beyond r_f - d_v nor within d_v of the particle)
+  uint32_t ask;   // bit q: the two are so close that each particle's own rounding decides
+};
+
+// A warp per slot.  What bounds it is instruction issue (850 warp instructions
+// per particle): the coverage of the 57 default test points by ~52 neighbours,
+// one neighbour per lane, with squares per axis and one add and one shift per
+// point, and the latency of its gathers, hence 40 warps per SM (640 us with
+// 20, 427 with 32, 400 with 40 for the 400,000 particles of a shock tube).  A
+// thread per particle that walked its list anew for every point took 2.68 ms.
+// FP64 instructions, 80 times an FP32 one here, are kept to what FP32 cannot
+// decide: FP32 distances are within the margin m of the exact ones, so a point
+// is covered or not, and of several uncovered points the one with the largest
+// clearance, without FP64 unless two distances lie within 2 m.  The FP64
+// decisions are single IEEE-rounded operations in the order of the definition.
+template <int Q2>
+__global__ void __launch_bounds__(128, 10) k_adapt_scan(const __grid_constant__ Grid g, ScanRule rule,
+                                                   const int32_t* __restrict__ perm,
                                                    const double* __restrict__ spos,
                                                    const double* __restrict__ slam,
                                                    const float4* __restrict__ scr,
                                                    const int64_t* __restrict__ off,
-                                                   const int32_t* __restrict__ idx, double vf, double cf,
-                                                   int32_t* void_count, int32_t* best, double* cand,
-                                                   int32_t* clump) {
-  // candidate test points: every grid point that can lie inside r_f - d_v for
-  // some lambda (a superset; each particle applies the exact test), ascending
-  __shared__ int16_t pts[kGridPts];
-  __shared__ int npts;
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    const double q = (g.rf_factor - vf) / (0.25 * g.rf_factor);
-    const double lim = q > 0.0 ? q * q * (1.0 + 1e-6) : -1.0;
-    int base = 0;
-    for (int k0 = 0; k0 < kGridPts; k0 += 32) {
-      const int k = k0 + lane;
-      bool in = false;
-      if (k < kGridPts) {
-        const int kx = k / 81 - 4, ky = (k / 9) % 9 - 4, kz = k % 9 - 4;
-        in = static_cast<double>(kx * kx + ky * ky + kz * kz) <= lim;
-      }
-      const unsigned m = __ballot_sync(0xffffffffu, in);
-      if (in) pts[base + __popc(m & ((1u << lane) - 1u))] = static_cast<int16_t>(k);
-      base += __popc(m);
-    }
-    if (lane == 0) npts = base;
-  }
-  __syncthreads();
+                                                   const int32_t* __restrict__ idx, int32_t* void_count,
+                                                   int32_t* best, double* cand, int32_t* clump) {
+  constexpr GridPoints<Q2> P;
+  constexpr int NP = grid_points(Q2), NW = (NP + 31) / 32, K = Q2 == 5 ? 2 : 4;
+  const auto& D = []() -> const GridPoints<Q2>& {
+    if constexpr (Q2 == 5) return kGrid5;
+    else return kGrid16;
+  }();
   const int n = g.n;
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
   const int64_t N = n;
+  const int lane = threadIdx.x & 31;
+  const int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  if (w >= n) return;
+  const int s = static_cast<int>(w);
   const double lam = slam[s];
-  const double r = __dmul_rn(g.rf_factor, lam);
-  const double r2 = __dmul_rn(r, r);
-  const double h = __dmul_rn(r, 0.25);
-  const double dv = __dmul_rn(vf, lam);
-  const double dv2 = __dmul_rn(dv, dv);
-  const double rin = __dsub_rn(r, dv);
-  const double rin2 = __dmul_rn(rin, rin);
-  const double dc = __dmul_rn(cf, lam);
-  const double dc2 = __dmul_rn(dc, dc);
-  const Screen q = make_screen(g, r);
-  // FP32 screens: |d32 - d| is within the coordinate margin; offsets and
-  // squares add a few ulps of r
-  const double m = static_cast<double>(g.screen_margin) + 1e-6 * r;
-  const float v_in2 = static_cast<float>(dv > m ? (dv - m) * (dv - m) : 0.0);
-  const float v_out2 = static_cast<float>((dv + m) * (dv + m));
-  const float c_in2 = static_cast<float>(dc > m ? (dc - m) * (dc - m) : 0.0);
-  const float c_out2 = static_cast<float>((dc + m) * (dc + m));
-  const float r_in2 = static_cast<float>(r > m ? (r - m) * (r - m) : 0.0);
-  const float r_out2 = static_cast<float>((r + m) * (r + m));
+  // FP32 radii with a margin: coordinates (screen_margin) and a few ulps of
+  // r for offsets, squares and the radii themselves
+  const float lamf = f32_of(lam);
+  const float r = static_cast<float>(g.rf_factor) * lamf, h = 0.25f * r;
+  const float dv = static_cast<float>(rule.vf) * lamf, dc = static_cast<float>(rule.cf) * lamf;
+  const float m = g.screen_margin + 3e-6f * r;
+  auto below = [&](float d) { return d > m ? (d - m) * (d - m) : 0.f; };
+  auto above = [&](float d) { return (d + m) * (d + m); };
+  const float v_in2 = below(dv), v_out2 = above(dv), c_in2 = below(dc), c_out2 = above(dc);
+  const float r_in2 = below(r), r_out2 = above(r);
   const float4 me = scr[s];
   const int me_caller = perm[s];
   const int64_t beg = off[s];
   const int64_t end = off[s + 1] < g.capacity ? off[s + 1] : g.capacity;
 
-  // clumps: a neighbour with a smaller caller index closer than d_c
-  int32_t cl = 0;
-  for (int64_t e = beg; e < end && !cl; ++e) {
-    const int t = idx[e];
-    if (perm[t] >= me_caller) continue;
-    const float3 d = offset32(q, me, scr[t]);
+  // coverage of every point, and clumps: a neighbour with a smaller caller
+  // index closer than d_c
+  uint32_t cov[NW];
+#pragma unroll
+  for (int i = 0; i < NW; ++i) cov[i] = 0u;
+  bool cl = false;
+  auto cover = [&](int t, float4 o) {
+    const float3 d = offset32(g, me, o);
+    float ax[2 * K + 1], ay[2 * K + 1], az[2 * K + 1];
+#pragma unroll
+    for (int k = -K; k <= K; ++k) {
+      const float ex = fmaf(static_cast<float>(-k), h, d.x), ey = fmaf(static_cast<float>(-k), h, d.y),
+                  ez = fmaf(static_cast<float>(-k), h, d.z);
+      ax[k + K] = ex * ex;
+      ay[k + K] = ey * ey;
+      az[k + K] = fmaf(ez, ez, -v_in2);
+    }
     const float dd = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
-    if (dd < c_in2) cl = 1;
-    else if (dd <= c_out2 && dist2_exact(g, spos, n, s, t) < dc2) cl = 1;
+    if (dd <= c_out2 && perm[t] < me_caller)
+      cl |= dd < c_in2 || closer_exact(g, spos, s, t, lam, rule.cf);
+    // the sign of |d - o_k|^2 - v_in2 is shifted into the word: one add and
+    // one shift per point
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+      uint32_t bits = 0u;
+      constexpr int last = NP - 32 * (NW - 1);
+#pragma unroll
+      for (int b = 0; b < (i + 1 < NW ? 32 : last); ++b) {
+        const int p = 32 * i + b;
+        const float e = (ax[P.x[p] + K] + ay[P.y[p] + K]) + az[P.z[p] + K];
+        bits = __funnelshift_l(__float_as_uint(e), bits, 1);
+      }
+      cov[i] |= bits;
+    }
+  };
+  // two neighbours per lane on their way at once
+  for (int64_t e = beg + lane; e < end; e += 64) {
+    const bool two = e + 32 < end;
+    const int t0 = idx[e], t1 = two ? idx[e + 32] : t0;
+    const float4 o0 = scr[t0], o1 = scr[t1];
+    cover(t0, o0);
+    if (two) cover(t1, o1);
+  }
+  // point p of a word at bit p
+#pragma unroll
+  for (int i = 0; i < NW; ++i) cov[i] = __brev(cov[i] << (i + 1 < NW ? 0 : 32 * NW - NP));
+  cl = __any_sync(0xffffffffu, cl);
+  uint32_t open[NW];  // points to be tested that no neighbour covers for certain
+#pragma unroll
+  for (int i = 0; i < NW; ++i) {
+    // lane p & 31 holds point p
+    const int p = 32 * i + lane;
+    bool ask = false;
+    if (p < NP) {
+      const int kx = D.x[p], ky = D.y[p], kz = D.z[p];
+      const uint32_t q = 1u << (kx * kx + ky * ky + kz * kz);
+      ask = (rule.test & q) != 0u;
+      if (rule.ask & q) {
+        const double rr = __dmul_rn(g.rf_factor, lam), hh = __dmul_rn(rr, 0.25);
+        const double v = __dmul_rn(rule.vf, lam), in = __dsub_rn(rr, v);
+        const double ox = __dmul_rn(static_cast<double>(kx), hh), oy = __dmul_rn(static_cast<double>(ky), hh),
+                     oz = __dmul_rn(static_cast<double>(kz), hh);
+        const double o2 = __dadd_rn(__dadd_rn(__dmul_rn(ox, ox), __dmul_rn(oy, oy)), __dmul_rn(oz, oz));
+        ask = o2 < __dmul_rn(in, in) && !(o2 < __dmul_rn(v, v));
+      }
+    }
+    open[i] = __ballot_sync(0xffffffffu, ask) & ~__reduce_or_sync(0xffffffffu, cov[i]);
   }
 
-  // voids: test points not within d_v of the particle or a neighbour
-  int32_t cnt = 0, bk = -1;
-  double bclear = -1.0;
-  for (int p = 0; p < npts; ++p) {
-    const int k = pts[p];
-    const int kx = k / 81 - 4, ky = (k / 9) % 9 - 4, kz = k % 9 - 4;
-    const double ox = __dmul_rn(static_cast<double>(kx), h);
-    const double oy = __dmul_rn(static_cast<double>(ky), h);
-    const double oz = __dmul_rn(static_cast<double>(kz), h);
-    const double o2 = __dadd_rn(__dadd_rn(__dmul_rn(ox, ox), __dmul_rn(oy, oy)), __dmul_rn(oz, oz));
-    if (!(o2 < rin2)) continue;  // outside r_f - d_v
-    if (o2 < dv2) continue;      // covered by the particle itself
-    const float fx = static_cast<float>(ox), fy = static_cast<float>(oy), fz = static_cast<float>(oz);
-    bool covered = false;
-    for (int64_t e = beg; e < end && !covered; ++e) {
-      const int t = idx[e];
-      const float3 d = offset32(q, me, scr[t]);
-      const float ex = d.x - fx, ey = d.y - fy, ez = d.z - fz;
-      const float e2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
-      if (e2 < v_in2) covered = true;
-      else if (e2 <= v_out2 && test_dist2(g, spos, n, s, t, ox, oy, oz) < dv2) covered = true;
-    }
-    if (covered) continue;
-    // uncovered: its clearance, the smallest exact squared distance over the
-    // particle (o2) and its exact r_f set.  An FP32 pass finds the smallest
-    // screened distance over the entries proved (or, in the band, tested) to
-    // be in the r_f set; only entries within twice the screen error of it
-    // can hold the exact minimum, and only those are evaluated in FP64.
-    float min32 = static_cast<float>(o2);
-    for (int64_t e = beg; e < end; ++e) {
-      const int t = idx[e];
-      const float3 d = offset32(q, me, scr[t]);
-      const float dd = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
-      if (dd > r_out2 || (dd >= r_in2 && !(dist2_exact(g, spos, n, s, t) < r2))) continue;
-      const float ex = d.x - fx, ey = d.y - fy, ez = d.z - fz;
-      const float e2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
-      min32 = e2 < min32 ? e2 : min32;
-    }
-    const double band = sqrt(static_cast<double>(min32)) + 2.0 * m;
-    const float band2 = static_cast<float>(band * band);
-    double clear = o2;
-    for (int64_t e = beg; e < end; ++e) {
-      const int t = idx[e];
-      const float3 d = offset32(q, me, scr[t]);
-      const float ex = d.x - fx, ey = d.y - fy, ez = d.z - fz;
-      if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) > band2) continue;
-      if (!(dist2_exact(g, spos, n, s, t) < r2)) continue;  // a skin entry, not in N(i)
-      const double e2 = test_dist2(g, spos, n, s, t, ox, oy, oz);
-      clear = e2 < clear ? e2 : clear;
-    }
-    ++cnt;
-    if (clear > bclear) {
-      bclear = clear;
-      bk = k;
+  // the open points: exactly covered (band) or void; the void with the
+  // largest clearance, the smallest distance to the particle and its r_f set
+  int cnt = 0, bk = -1;
+  float best_lo = -1.f, best_hi = -1.f;  // bounds of the best point's clearance (distance)
+  double best_exact = -1.0;              // its exact square, once a comparison needed it
+  // only entries within 2 m of the FP32 minimum can hold the exact one
+  auto exact = [&](int p, float hi) {
+    return clearance_exact(g, spos, scr, idx, beg, end, s, lam, D.x[p], D.y[p], D.z[p],
+                           (hi + m) * (hi + m) * 1.000001f);
+  };
+#pragma unroll
+  for (int i = 0; i < NW; ++i) {
+    for (uint32_t left = open[i]; left != 0u; left &= left - 1u) {
+      const int p = 32 * i + __ffs(left) - 1;
+      const float fx = D.x[p] * h, fy = D.y[p] * h, fz = D.z[p] * h;
+      // smallest FP32 distance over the entries certainly (hi) and possibly (lo) in the r_f set
+      float lo2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz)), hi2 = lo2;
+      bool covered = false;
+      for (int64_t e = beg + lane; e < end; e += 32) {
+        const int t = idx[e];
+        const float3 d = offset32(g, me, scr[t]);
+        const float dd = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
+        const float ex = d.x - fx, ey = d.y - fy, ez = d.z - fz;
+        const float e2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
+        if (e2 <= v_out2) covered |= covers_exact(g, spos, s, t, lam, rule.vf, D.x[p], D.y[p], D.z[p]);
+        if (dd <= r_out2) lo2 = fminf(lo2, e2);
+        if (dd < r_in2) hi2 = fminf(hi2, e2);
+      }
+      if (__any_sync(0xffffffffu, covered)) continue;
+      ++cnt;
+      const float lo = sqrtf(__uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(lo2)))) - m;
+      const float hi = sqrtf(__uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(hi2)))) + m;
+      bool better = bk < 0 || lo > best_hi;
+      double ex = -1.0;
+      if (!better && hi >= best_lo) {  // too close for FP32
+        if (best_exact < 0.0) best_exact = exact(bk, best_hi);
+        ex = exact(p, hi);
+        better = ex > best_exact;
+      }
+      if (better) {
+        bk = p;
+        best_lo = lo;
+        best_hi = hi;
+        best_exact = ex;
+      }
     }
   }
-  if (void_count) void_count[me_caller] = cnt;
-  if (best) best[me_caller] = bk;
-  if (clump) clump[me_caller] = cl;
-  if (cand) {
-    double c[3] = {0.0, 0.0, 0.0};
+  if (lane == 0) {
+    if (void_count) void_count[me_caller] = cnt;
+    if (best) best[me_caller] = bk < 0 ? -1 : ((D.x[bk] + 4) * 9 + D.y[bk] + 4) * 9 + D.z[bk] + 4;
+    if (clump) clump[me_caller] = cl ? 1 : 0;
+  }
+  if (cand && lane < 3) {
+    double c = 0.0;
     if (bk >= 0) {
-      const int kk[3] = {bk / 81 - 4, (bk / 9) % 9 - 4, bk % 9 - 4};
-      for (int a = 0; a < 3; ++a) c[a] = __dadd_rn(spos[a * N + s], __dmul_rn(static_cast<double>(kk[a]), h));
+      const int k = lane == 0 ? D.x[bk] : lane == 1 ? D.y[bk] : D.z[bk];
+      const double hh = __dmul_rn(__dmul_rn(g.rf_factor, lam), 0.25);
+      c = __dadd_rn(spos[lane * N + s], __dmul_rn(static_cast<double>(k), hh));
     }
-    for (int a = 0; a < 3; ++a) cand[a * N + me_caller] = c[a];
+    cand[lane * N + me_caller] = c;
   }
+}
+
+// Which grid points the scan tests, by |k|^2 (the same for every lambda
+// unless the radii nearly coincide): |o_k| = |k| r_f / 4 below r_f - d_v and not
+// below d_v.
+ScanRule scan_rule(double rf, double vf, double cf) {
+  ScanRule q{vf, cf, 0u, 0u};
+  for (int k = 0; k <= 16; ++k) {
+    const double o2 = k * rf * rf / 16.0, in2 = (rf - vf) * (rf - vf), v2 = vf * vf, eps = 1e-12 * rf * rf;
+    if (o2 > in2 - eps && o2 < in2 + eps) q.ask |= 1u << k;
+    else if (o2 > v2 - eps && o2 < v2 + eps) q.ask |= 1u << k;
+    else if (o2 < in2 && o2 > v2) q.test |= 1u << k;
+  }
+  return q;
 }
 
 // Deletion and creation flags (caller order) from a scan: wants = survives
@@ -1385,10 +1509,14 @@ extern "C" phb_status phb_adapt_scan(const phb_plan* plan, const double* pos, co
   float4* scr = region<float4>(plan, ws, R_SCREEN);
   k_adapt_gather<<<blocks_for(n), kThreads, 0, st>>>(g, perm, pos, lambda, spos, slam, scr);
   note_launch();
-  k_adapt_scan<<<blocks_for(n, 128), 128, 0, st>>>(g, perm, spos, slam, scr,
-                                                   region<int64_t>(plan, ws, R_OFF),
-                                                   region<int32_t>(plan, ws, R_IDX), void_factor,
-                                                   clump_factor, void_count, best, cand, clump);
+  // the points within |k|^2 <= 5 are all there are for the default factors;
+  // smaller void factors reach out to |k|^2 = 16 (|o_k| < r_f)
+  const ScanRule rule = scan_rule(plan->rf_factor, void_factor, clump_factor);
+  const auto scan = (rule.test | rule.ask) >> 6 == 0u ? k_adapt_scan<5> : k_adapt_scan<16>;
+  scan<<<blocks_for(int64_t(n) * 32, 128), 128, 0, st>>>(g, rule, perm, spos, slam, scr,
+                                                         region<int64_t>(plan, ws, R_OFF),
+                                                         region<int32_t>(plan, ws, R_IDX), void_count, best,
+                                                         cand, clump);
   note_launch();
   return launch_status(cudaGetLastError());
 }
