@@ -49,17 +49,58 @@ __global__ void k_scatter(int n, const int32_t* __restrict__ keys, const int32_t
 // Make the order inside each cell deterministic: ascending caller index.
 // Thread per particle: its rank among the particles of its cell is the number
 // of them with a smaller caller index (the cells' members come from the
-// atomic scatter in arbitrary order).
-__global__ void k_rank_cells(int n, const int32_t* __restrict__ keys,
-                             const int32_t* __restrict__ cell_start,
-                             const int32_t* __restrict__ scattered, int32_t* __restrict__ perm) {
+// atomic scatter in arbitrary order).  That is quadratic in a cell's members
+// (~12), so a cell of more than kBigCell - a clump, or the particles without a
+// finite position, which all go to cell 0 - is listed in one sweep of the
+// block that holds its first scattered member.
+constexpr int kBigCell = 2048;
+
+__global__ void __launch_bounds__(kThreads) k_rank_cells(int n, const int32_t* __restrict__ keys,
+                                                         const int32_t* __restrict__ cell_start,
+                                                         const int32_t* __restrict__ scattered,
+                                                         int32_t* __restrict__ perm) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int32_t k = keys[i];
-  const int a = cell_start[k], b = cell_start[k + 1];
-  int rank = 0;
-  for (int t = a; t < b; ++t) rank += scattered[t] < i ? 1 : 0;
-  perm[a + rank] = i;
+  bool lead = false;
+  int32_t k = -1;
+  if (i < n) {
+    k = keys[i];
+    const int a = cell_start[k], b = cell_start[k + 1];
+    if (b - a <= kBigCell) {
+      int rank = 0;
+      for (int t = a; t < b; ++t) rank += scattered[t] < i ? 1 : 0;
+      perm[a + rank] = i;
+    } else {
+      lead = scattered[a] == i;
+    }
+  }
+  if (!__syncthreads_or(lead)) return;
+  __shared__ int cell;
+  __shared__ int sums[kThreads / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  while (__syncthreads_or(lead)) {
+    if (threadIdx.x == 0) cell = -1;
+    __syncthreads();
+    if (lead) atomicMax(&cell, k);
+    __syncthreads();
+    const int c = cell;
+    if (k == c) lead = false;
+    int at = cell_start[c];
+    for (int j0 = 0; j0 < n; j0 += kThreads) {
+      const int j = j0 + threadIdx.x;
+      const bool in = j < n && keys[j] == c;
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (lane == 0) sums[wid] = __popc(m);
+      __syncthreads();
+      int before = 0, total = 0;
+      for (int w = 0; w < kThreads / 32; ++w) {
+        before += w < wid ? sums[w] : 0;
+        total += sums[w];
+      }
+      if (in) perm[at + before + __popc(m & ((1u << lane) - 1u))] = j;
+      at += total;
+      __syncthreads();
+    }
+  }
 }
 
 // Slot-order copies of positions and lambda, the inverse permutation and the
@@ -185,8 +226,7 @@ __device__ __forceinline__ Screen make_screen(const Grid& g, double r) {
   return q;
 }
 
-// FP32 screen distance squared (the same arithmetic as is_neighbour): below
-// q.in2 a neighbour, above q.out2 not, in between the exact test decides.
+// FP32 screen distance squared: below q.in2 a neighbour, above q.out2 not, in between the exact test decides.
 template <bool kWrap>
 __device__ __forceinline__ float screen_d2(const Screen& q, float4 me, float4 o) {
   float dx = o.x - me.x, dy = o.y - me.y, dz = o.z - me.z;
@@ -196,21 +236,6 @@ __device__ __forceinline__ float screen_d2(const Screen& q, float4 me, float4 o)
     dz = fmaf(-q.lenf[2], rintf(dz * q.invlf[2]), dz);
   }
   return fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-}
-
-template <bool kWrap>
-__device__ __forceinline__ bool is_neighbour(const Grid& g, const Screen& q, const double* spos,
-                                             int s, int t, float4 me, float4 o) {
-  float dx = o.x - me.x, dy = o.y - me.y, dz = o.z - me.z;
-  if (kWrap) {
-    dx = fmaf(-q.lenf[0], rintf(dx * q.invlf[0]), dx);
-    dy = fmaf(-q.lenf[1], rintf(dy * q.invlf[1]), dy);
-    dz = fmaf(-q.lenf[2], rintf(dz * q.invlf[2]), dz);
-  }
-  const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  if (d2 < q.in2) return true;
-  if (d2 > q.out2) return false;
-  return dist2_exact(g, spos, g.n, s, t) < q.r2;
 }
 
 // Whether every cell of the reach on axis a lies inside the grid without
@@ -223,104 +248,37 @@ __device__ __forceinline__ bool plain_axis(const Grid& g, int a, int c, const Re
   return q.wrap && c - R >= 0 && c + R < g.ncell[a] && 2 * R + 3 <= g.ncell[a];
 }
 
-enum SearchOut { kCount = 0, kFillCsr = 1, kFillEll = 2 };
-
-// Cell culling for the cell-by-cell search of reaches that cover a whole
-// periodic axis (the run search does not cull): the reach box of 2R+1 cells
-// per axis is cut to the cells that can hold a point within r of the
-// particle.  With f the particle's
-// fractional position in its cell, the nearest point of the cell at offset i
-// is (i - f) cells away for i > 0, (-i - 1 + f) for i < 0 and 0 for i = 0.
-// Distances are taken with a margin of 1e-3 cells plus the screen margin, so
-// that only cells that cannot hold a neighbour are skipped; an axis whose
-// reach covers the whole periodic grid is not culled.
-struct Cull {
-  float f[3];      // fractional position in the cell, clamped to [0, 1]
-  float cell[3];   // cell edges
-  float rr;        // (r + margin)^2
-  bool on[3];      // axis culled
-};
-
-__device__ __forceinline__ float cull_d(const Cull& k, int a, int i) {
-  if (!k.on[a] || i == 0) return 0.f;
-  const float d = i > 0 ? i - k.f[a] : -i - 1 + k.f[a];
-  return d > 0.f ? d * k.cell[a] : 0.f;
+// The z cells of a reach as up to two runs of cells [a0, b0], [a1, b1] in the
+// order of the reach offsets; returns how many.
+__device__ __forceinline__ int z_runs(const Reach& qz, int ncz, int& a0, int& b0, int& a1, int& b1) {
+  const int za = qz.start, zb = qz.start + qz.count - 1;
+  a0 = za;
+  b0 = zb;
+  a1 = 0;
+  b1 = -1;
+  if (!qz.wrap) {
+    a0 = max(za, 0);
+    b0 = min(zb, ncz - 1);
+  } else if (za < 0) {  // wraps below: cells ncz + za .., then 0 .. zb
+    a0 = za + ncz;
+    b0 = zb < 0 ? zb + ncz : ncz - 1;
+    b1 = zb < 0 ? -1 : zb;
+  } else if (zb >= ncz) {  // wraps above: cells za .. ncz - 1, then 0 .. zb - ncz
+    a0 = za < ncz ? za : za - ncz;
+    b0 = za < ncz ? ncz - 1 : zb - ncz;
+    b1 = za < ncz ? zb - ncz : -1;
+  }
+  const int nseg = (a0 <= b0 ? 1 : 0) + (a1 <= b1 ? 1 : 0);
+  if (a0 > b0) {
+    a0 = a1;
+    b0 = b1;
+  }
+  return nseg;
 }
 
-__device__ __forceinline__ Cull make_cull(const Grid& g, const double* spos, int s, const int (&c)[3],
-                                          const Reach& qx, const Reach& qy, const Reach& qz, double r) {
-  Cull k;
-  const Reach* q[3] = {&qx, &qy, &qz};
-  double mc = 0.0;
-  for (int a = 0; a < 3; ++a) {
-    const double u = (spos[a * g.n + s] - g.lo[a]) * g.inv_cell[a];
-    const double f = g.periodic[a] ? u - floor(u) : u - c[a];
-    k.f[a] = static_cast<float>(f < 0.0 ? 0.0 : (f > 1.0 ? 1.0 : f));
-    k.cell[a] = static_cast<float>(g.cell[a]);
-    k.on[a] = !(g.periodic[a] && !q[a]->wrap);  // not the whole-axis reach
-    mc = g.cell[a] > mc ? g.cell[a] : mc;
-  }
-  const double rm = r + 1e-3 * mc + static_cast<double>(g.screen_margin);
-  k.rr = static_cast<float>(rm * rm);
-  return k;
-}
-
-// One particle's list: candidates from the culled cells within reach, looked
-// up through the linear (first slot, count) table, in cell order (x, y, z)
-// and slot order inside a cell.  kCount only counts; kFillCsr writes entries
-// [base, end) of the CSR lists; kFillEll writes the first g.ell entries to
-// the slot's row of the single-pass scratch.  Returns the exact count.
-template <int OUT, bool kWrap>
-__device__ int search_one(const Grid& g, const int2* __restrict__ clin, const float4* __restrict__ scr,
-                          const double* __restrict__ spos, const Screen& q, const Cull& cu,
-                          const Reach& qx, const Reach& qy, const Reach& qz, int s, int64_t base,
-                          int64_t end, int32_t* __restrict__ out) {
-  const float4 me = scr[s];
-  const int Rx = qx.count / 2, Ry = qy.count / 2, Rz = qz.count / 2;
-  int count = 0;
-  for (int kx = 0; kx < qx.count; ++kx) {
-    bool okx;
-    const int cx = axis_cell(g, 0, qx, kx, okx);
-    if (!okx) continue;
-    const float dx = cull_d(cu, 0, kx - Rx);
-    const float rx = cu.rr - dx * dx;
-    if (rx < 0.f) continue;
-    for (int ky = 0; ky < qy.count; ++ky) {
-      bool oky;
-      const int cy = axis_cell(g, 1, qy, ky, oky);
-      if (!oky) continue;
-      const float dy = cull_d(cu, 1, ky - Ry);
-      const float ry = rx - dy * dy;
-      if (ry < 0.f) continue;
-      // z cells within reach of this row
-      int z0 = 0, z1 = qz.count - 1;
-      if (cu.on[2]) {
-        const float sz = sqrtf(ry) / cu.cell[2];
-        const int hi = static_cast<int>(floorf(sz + cu.f[2]));
-        const int lo = -static_cast<int>(floorf(sz + 1.f - cu.f[2]));
-        z0 = max(0, lo + Rz);
-        z1 = min(qz.count - 1, hi + Rz);
-      }
-      const int64_t row = (static_cast<int64_t>(cx) * g.ncell[1] + cy) * g.ncell[2];
-      for (int kz = z0; kz <= z1; ++kz) {
-        bool okz;
-        const int cz = axis_cell(g, 2, qz, kz, okz);
-        if (!okz) continue;
-        const int2 sc = clin[row + cz];
-        for (int t = sc.x; t < sc.x + sc.y; ++t) {
-          if (t == s || !is_neighbour<kWrap>(g, q, spos, s, t, me, scr[t])) continue;
-          if (OUT == kFillCsr) {
-            const int64_t e = base + count;
-            if (e < g.capacity && e < end) out[e] = t;
-          } else if (OUT == kFillEll) {
-            if (count < g.ell) out[count] = t;
-          }
-          ++count;
-        }
-      }
-    }
-  }
-  return count;
+// A wrapped screen position that can have neighbours (finite, in FP32 too).
+__device__ __forceinline__ bool on_screen(float4 p) {
+  return fabsf(p.x) + fabsf(p.y) + fabsf(p.z) < __int_as_float(0x7f800000);
 }
 
 // Candidate records in linear cell order (k_fill_lin) and the cells' starts.
@@ -329,27 +287,22 @@ struct Lin {
   const int32_t* __restrict__ start;
 };
 
-// The same list as search_one (cells in x, y, z order of the reach box,
-// slot order inside a cell), for reaches that do not cover a whole periodic
-// axis: the z cells of one (x, y) row are read as one run of the linear-order
-// records (two where the row wraps a periodic z boundary), four candidates
-// per batch so that their loads overlap.  The reach box is not culled per
-// particle: the particles of one cell then walk identical rows and runs, so a
-// warp's lanes stay together (measured faster than culling, which skips ~20%
-// of the candidates but leaves half the lanes idle).
-template <int OUT, bool kWrap>
+// One particle's list by one thread: cells in x, y, z order of the reach box,
+// slot order inside a cell.  The z cells of one (x, y) row are read as one run
+// of the linear-order records (two where the row wraps a periodic z boundary),
+// four candidates per batch so that their loads overlap.  The reach box is not
+// culled per particle: the particles of one cell then walk identical rows and
+// runs, so a warp's lanes stay together (measured faster than culling, which
+// skips ~20% of the candidates but leaves half the lanes idle).  Writes the
+// first g.ell entries to out; returns the exact count.
+template <bool kWrap>
 __device__ int search_runs(const Grid& g, const Lin& lin, const double* __restrict__ spos,
                            const Screen& q, const Reach& qx, const Reach& qy, const Reach& qz,
-                           float4 me, int s, int64_t base, int64_t end, int32_t* __restrict__ out) {
+                           float4 me, int s, int32_t* __restrict__ out) {
   const int ncz = g.ncell[2];
   int count = 0;
   auto take = [&](int t) {
-    if (OUT == kFillCsr) {
-      const int64_t e = base + count;
-      if (e < g.capacity && e < end) out[e] = t;
-    } else if (OUT == kFillEll) {
-      if (count < g.ell) out[count] = t;
-    }
+    if (count < g.ell) out[count] = t;
     ++count;
   };
   for (int kx = 0; kx < qx.count; ++kx) {
@@ -360,23 +313,8 @@ __device__ int search_runs(const Grid& g, const Lin& lin, const double* __restri
       bool oky;
       const int cy = axis_cell(g, 1, qy, ky, oky);
       if (!oky) continue;
-      int za = qz.start, zb = qz.start + qz.count - 1;
-      // up to two runs of cells [a0, b0], [a1, b1], in the order of the reach offsets
-      int a0 = za, b0 = zb, a1 = 0, b1 = -1;
-      if (!qz.wrap) {
-        a0 = max(za, 0);
-        b0 = min(zb, ncz - 1);
-      } else if (za < 0) {  // wraps below: cells ncz + za .., then 0 .. zb
-        a0 = za + ncz;
-        b0 = zb < 0 ? zb + ncz : ncz - 1;
-        b1 = zb < 0 ? -1 : zb;
-      } else if (zb >= ncz) {  // wraps above: cells za .. ncz - 1, then 0 .. zb - ncz
-        a0 = za < ncz ? za : za - ncz;
-        b0 = za < ncz ? ncz - 1 : zb - ncz;
-        b1 = za < ncz ? zb - ncz : -1;
-      }
-      const int nseg = (a0 <= b0 ? 1 : 0) + (a1 <= b1 ? 1 : 0);
-      if (a0 > b0) { a0 = a1; b0 = b1; }
+      int a0, b0, a1, b1;
+      const int nseg = z_runs(qz, ncz, a0, b0, a1, b1);
       const int64_t row = (static_cast<int64_t>(cx) * g.ncell[1] + cy) * ncz;
       for (int k = 0; k < nseg; ++k) {
         const int t0 = lin.start[row + (k == 0 ? a0 : a1)];
@@ -419,41 +357,128 @@ __device__ int search_runs(const Grid& g, const Lin& lin, const double* __restri
   return count;
 }
 
-template <int OUT>
-__device__ int search_particle(const Grid& g, const int2* __restrict__ clin, const Lin& lin,
-                               const int32_t* __restrict__ cellc, const float4* __restrict__ scr,
-                               const double* __restrict__ spos, double r, int s, int64_t base,
-                               int64_t end, int32_t* __restrict__ out) {
-  const Screen q = make_screen(g, r);
-  int c[3];
-  unpack_cell(cellc[s], c[0], c[1], c[2]);
-  const Reach qx = axis_reach(g, 0, c[0], r);
-  const Reach qy = axis_reach(g, 1, c[1], r);
-  const Reach qz = axis_reach(g, 2, c[2], r);
-  const bool plain =
-      plain_axis(g, 0, c[0], qx) && plain_axis(g, 1, c[1], qy) && plain_axis(g, 2, c[2], qz);
-  // a periodic axis whose reach is the whole axis has no wrap flag
-  const bool whole = (g.periodic[0] && !qx.wrap) || (g.periodic[1] && !qy.wrap) ||
-                     (g.periodic[2] && !qz.wrap);
-  if (!whole) {
-    const float4 me = scr[s];
-    if (plain) return search_runs<OUT, false>(g, lin, spos, q, qx, qy, qz, me, s, base, end, out);
-    return search_runs<OUT, true>(g, lin, spos, q, qx, qy, qz, me, s, base, end, out);
+__device__ __forceinline__ int warp_excl_scan(int v, int lane) {
+  int x = v;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, d);
+    if (lane >= d) x += y;
   }
-  // a reach covering a whole periodic axis: cell by cell, culled
-  const Cull cu = make_cull(g, spos, s, c, qx, qy, qz, r);
-  if (plain) return search_one<OUT, false>(g, clin, scr, spos, q, cu, qx, qy, qz, s, base, end, out);
-  return search_one<OUT, true>(g, clin, scr, spos, q, cu, qx, qy, qz, s, base, end, out);
+  return x - v;
 }
 
-// The CSR fill of one list longer than the scratch rows (rare): kept out of
-// line so that it does not weigh on the compaction kernel's registers.
-__device__ __noinline__ void search_overflow(const Grid& g, const int2* __restrict__ clin, Lin lin,
-                                             const int32_t* __restrict__ cellc,
+// One particle's list by one warp: the same candidates in the same order, the
+// runs of 32 rows at a time laid out as one sequence, 32 candidates per chunk,
+// a ballot appending the hits.  Entries to out[0 .. room); returns the exact
+// count.  table: 2 x 64 + 1 ints of the warp's shared memory.  rx, ry, rz: reach in cells.
+constexpr int kWarpTable = 2 * 64 + 1;
+template <bool kWrap>
+__device__ __forceinline__ int search_rows(const Grid& g, const Lin& lin, const double* __restrict__ spos,
+                                           float in2, float out2, double r2, const Reach& qx,
+                                           const Reach& qy, const Reach& qz, float4 me, int s, int* table,
+                                           int64_t room, int32_t* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  int* t0 = table;         // first linear-order record of each run
+  int* pre = table + 64;   // candidates before each run (the last: the total)
+  const int ncy = g.ncell[1], ncz = g.ncell[2];
+  const int nrow = qx.count * qy.count;
+  int count = 0;
+  Screen q;
+  for (int a = 0; a < 3; ++a) {
+    q.lenf[a] = g.lenf[a];
+    q.invlf[a] = g.inv_lenf[a];
+  }
+  for (int j0 = 0; j0 < nrow; j0 += 32) {
+    const int j = j0 + lane;
+    int nr = 0, ta = 0, la = 0, tb = 0, lb = 0;
+    if (j < nrow) {
+      const int kx = j / qy.count, ky = j - kx * qy.count;
+      bool okx, oky;
+      const int rx = axis_cell(g, 0, qx, kx, okx), ry = axis_cell(g, 1, qy, ky, oky);
+      if (okx && oky) {
+        int a0, b0, a1, b1;
+        nr = z_runs(qz, ncz, a0, b0, a1, b1);
+        const int64_t row = (static_cast<int64_t>(rx) * ncy + ry) * ncz;
+        if (nr >= 1) {
+          ta = lin.start[row + a0];
+          la = lin.start[row + b0 + 1] - ta;
+        }
+        if (nr == 2) {
+          tb = lin.start[row + a1];
+          lb = lin.start[row + b1 + 1] - tb;
+        }
+      }
+    }
+    const int rpos = warp_excl_scan(nr, lane), cpos = warp_excl_scan(la + lb, lane);
+    if (nr >= 1) {
+      t0[rpos] = ta;
+      pre[rpos] = cpos;
+    }
+    if (nr == 2) {
+      t0[rpos + 1] = tb;
+      pre[rpos + 1] = cpos + la;
+    }
+    const int nrun = __shfl_sync(0xffffffffu, rpos + nr, 31);
+    const int total = __shfl_sync(0xffffffffu, cpos + la + lb, 31);
+    if (lane == 0) pre[nrun] = total;
+    __syncwarp();
+    int run = 0;  // the run holding the next chunk's first candidate
+    auto fetch = [&](int v0) {
+      const int v = v0 + lane;
+      float4 o = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, __int_as_float(-1));
+      int rn = run;
+      if (v < total) {
+        while (pre[rn + 1] <= v) ++rn;
+        o = lin.rec[t0[rn] + (v - pre[rn])];
+      }
+      run = __shfl_sync(0xffffffffu, rn, 31);
+      return o;
+    };
+    float4 next = fetch(0);
+    for (int v0 = 0; v0 < total; v0 += 32) {
+      const float4 o = next;
+      if (v0 + 32 < total) next = fetch(v0 + 32);  // one chunk ahead
+      const int t = __float_as_int(o.w);
+      const float d = screen_d2<kWrap>(q, me, o);
+      bool hit = t != s && d < in2;
+      if (t != s && !hit && d <= out2) hit = dist2_exact(g, spos, g.n, s, t) < r2;
+      const unsigned m = __ballot_sync(0xffffffffu, hit);
+      if (hit) {
+        const int e = count + __popc(m & ((1u << lane) - 1u));
+        if (e < room) out[e] = t;
+      }
+      count += __popc(m);
+    }
+    __syncwarp();  // the next rows rewrite the table
+  }
+  return count;
+}
+
+__device__ __forceinline__ int search_warp(const Grid& g, const Lin& lin, const double* __restrict__ spos,
+                                           float in2, float out2, double r2, int rx, int ry, int rz,
+                                           int32_t cell, float4 me, int s, int* table, int64_t room,
+                                           int32_t* __restrict__ out) {
+  if (!on_screen(me)) return 0;
+  int c[3];
+  unpack_cell(cell, c[0], c[1], c[2]);
+  const Reach qx = axis_reach_cells(g, 0, c[0], rx);
+  const Reach qy = axis_reach_cells(g, 1, c[1], ry);
+  const Reach qz = axis_reach_cells(g, 2, c[2], rz);
+  if (plain_axis(g, 0, c[0], qx) && plain_axis(g, 1, c[1], qy) && plain_axis(g, 2, c[2], qz))
+    return search_rows<false>(g, lin, spos, in2, out2, r2, qx, qy, qz, me, s, table, room, out);
+  return search_rows<true>(g, lin, spos, in2, out2, r2, qx, qy, qz, me, s, table, room, out);
+}
+
+// The CSR fill of one list longer than the scratch rows, by one warp (rare):
+// kept out of line so that it does not weigh on the compaction kernel's
+// registers.
+__device__ __noinline__ void search_overflow(const Grid& g, Lin lin, const int32_t* __restrict__ cellc,
                                              const float4* __restrict__ scr,
-                                             const double* __restrict__ spos, double r, int s,
-                                             int64_t base, int64_t end, int32_t* __restrict__ out) {
-  search_particle<kFillCsr>(g, clin, lin, cellc, scr, spos, r, s, base, end, out);
+                                             const double* __restrict__ spos, double r, int s, int* table,
+                                             int64_t room, int32_t* __restrict__ out) {
+  const Screen q = make_screen(g, r);
+  search_warp(g, lin, spos, q.in2, q.out2, q.r2, reach_cells(g, 0, r), reach_cells(g, 1, r),
+              reach_cells(g, 2, r), cellc[s], scr[s], s, table, room, out);
 }
 
 constexpr int kRunCap = 128;  // candidate runs a warp records (a reach of 3 cells: at most 98)
@@ -475,16 +500,6 @@ static_assert(offsetof(SearchWarp, nx) % 16 == 0 && offsetof(SearchWarp, ny) % 1
                   offsetof(SearchWarp, nz) % 16 == 0 && offsetof(SearchWarp, in2) % 16 == 0 &&
                   offsetof(SearchWarp, out2) % 16 == 0 && offsetof(SearchWarp, slot) % 16 == 0,
               "vector-read arrays of SearchWarp must be 16-byte aligned");
-
-__device__ __forceinline__ int warp_excl_scan(int v, int lane) {
-  int x = v;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, d);
-    if (lane >= d) x += y;
-  }
-  return x - v;
-}
 
 // Squared FP32 screen distances of candidate o to two homes (a, b): packed
 // FP32x2, each half rounded as screen_d2 rounds it.
@@ -594,6 +609,10 @@ __global__ void __launch_bounds__(32, 32) k_search_cells(Grid g, Lin lin,
     float4 me = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
     if (mine) me = lin.rec[g0 + lane];
     const int s = __float_as_int(me.w);
+    if (__all_sync(0xffffffffu, !mine || !on_screen(me))) {  // no positions: no neighbours
+      if (mine) ncnt[s] = 0;
+      continue;
+    }
     double r = 0.0;
     int R[3] = {0, 0, 0};
     if (mine) {
@@ -625,22 +644,8 @@ __global__ void __launch_bounds__(32, 32) k_search_cells(Grid g, Lin lin,
         const int rx = axis_cell(g, 0, qx, kx, okx);
         const int ry = axis_cell(g, 1, qy, ky, oky);
         if (okx && oky) {
-          const int za = qz.start, zb = qz.start + qz.count - 1;
-          int a0 = za, b0 = zb, a1 = 0, b1 = -1;
-          if (!qz.wrap) {
-            a0 = max(za, 0);
-            b0 = min(zb, ncz - 1);
-          } else if (za < 0) {
-            a0 = za + ncz;
-            b0 = zb < 0 ? zb + ncz : ncz - 1;
-            b1 = zb < 0 ? -1 : zb;
-          } else if (zb >= ncz) {
-            a0 = za < ncz ? za : za - ncz;
-            b0 = za < ncz ? ncz - 1 : zb - ncz;
-            b1 = za < ncz ? zb - ncz : -1;
-          }
-          nr = (a0 <= b0 ? 1 : 0) + (a1 <= b1 ? 1 : 0);
-          if (a0 > b0) { a0 = a1; b0 = b1; }
+          int a0, b0, a1, b1;
+          nr = z_runs(qz, ncz, a0, b0, a1, b1);
           const int64_t row = (static_cast<int64_t>(rx) * ncy + ry) * ncz;
           if (nr >= 1) {
             ta = lin.start[row + a0];
@@ -720,8 +725,7 @@ __global__ void __launch_bounds__(32, 32) k_search_cells(Grid g, Lin lin,
 // Single pass, thread per particle (slot order): exact list lengths and the
 // first g.ell entries of every list (after the cell-major search, left_only:
 // of the lists it left, ncnt still -1).
-__global__ void __launch_bounds__(kThreads, 4) k_search_ell(Grid g, const int2* __restrict__ clin,
-                                                         Lin lin, const int32_t* __restrict__ cellc,
+__global__ void __launch_bounds__(kThreads, 4) k_search_ell(Grid g, Lin lin, const int32_t* __restrict__ cellc,
                                                          const float4* __restrict__ scr,
                                                          const double* __restrict__ spos,
                                                          const double* __restrict__ slam,
@@ -731,9 +735,60 @@ __global__ void __launch_bounds__(kThreads, 4) k_search_ell(Grid g, const int2* 
   if (s >= g.n) return;
   if (s == g.n - 1) ncnt[g.n] = 0;  // the offsets scan's sentinel
   if (left_only && ncnt[s] >= 0) return;
+  const float4 me = scr[s];
+  if (!on_screen(me)) {
+    ncnt[s] = 0;
+    return;
+  }
   const double r = list_radius(g, slam[s]);
-  ncnt[s] = search_particle<kFillEll>(g, clin, lin, cellc, scr, spos, r, s, 0, 0,
-                                      ell + static_cast<int64_t>(s) * g.ell);
+  const Screen q = make_screen(g, r);
+  int c[3];
+  unpack_cell(cellc[s], c[0], c[1], c[2]);
+  const Reach qx = axis_reach(g, 0, c[0], r);
+  const Reach qy = axis_reach(g, 1, c[1], r);
+  const Reach qz = axis_reach(g, 2, c[2], r);
+  int32_t* out = ell + static_cast<int64_t>(s) * g.ell;
+  const bool plain =
+      plain_axis(g, 0, c[0], qx) && plain_axis(g, 1, c[1], qy) && plain_axis(g, 2, c[2], qz);
+  ncnt[s] = plain ? search_runs<false>(g, lin, spos, q, qx, qy, qz, me, s, out)
+                  : search_runs<true>(g, lin, spos, q, qx, qy, qz, me, s, out);
+}
+
+// The same by a warp per particle, for sets too small to fill the GPU with
+// threads (40 blocks hold 10,007 particles).  Two particles per warp: their
+// FP64 set-up (28 instructions, 20 SM cycles each per warp) runs once for
+// both, a lane each (eight: 66 instead of 38 us for 10,007 particles, 123
+// instead of 116 for 60,000: too few warps).
+__global__ void __launch_bounds__(128) k_search_warp(Grid g, Lin lin, const int32_t* __restrict__ cellc,
+                                                     const float4* __restrict__ scr,
+                                                     const double* __restrict__ spos,
+                                                     const double* __restrict__ slam,
+                                                     int32_t* __restrict__ ncnt, int32_t* __restrict__ ell) {
+  constexpr int kPairs = 2;
+  __shared__ int table[4][kWarpTable];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t s0 = (static_cast<int64_t>(blockIdx.x) * 4 + wid) * kPairs;
+  if (s0 >= g.n) return;
+  const int last = g.n - 1;
+  const int mine = static_cast<int>(s0 + lane % kPairs < g.n ? s0 + lane % kPairs : last);
+  const double r = list_radius(g, slam[mine]);
+  const Screen q = make_screen(g, r);
+  const int rx = reach_cells(g, 0, r), ry = reach_cells(g, 1, r), rz = reach_cells(g, 2, r);
+  const int32_t cell = cellc[mine];
+  const float4 me = scr[mine];
+  const bool todo = lane < kPairs && s0 + lane < g.n;
+  int count = 0;
+  for (unsigned left = __ballot_sync(0xffffffffu, todo); left != 0u; left &= left - 1u) {
+    const int p = __ffs(left) - 1;
+    auto of = [&](auto v) { return __shfl_sync(0xffffffffu, v, p); };
+    const int s = of(mine);
+    const int c = search_warp(g, lin, spos, of(q.in2), of(q.out2), of(q.r2), of(rx), of(ry), of(rz), of(cell),
+                              make_float4(of(me.x), of(me.y), of(me.z), 0.f), s, table[wid], g.ell,
+                              ell + static_cast<int64_t>(s) * g.ell);
+    if (lane == p) count = c;
+  }
+  if (todo) ncnt[mine] = count;
+  if (lane < kPairs && s0 + lane == last) ncnt[g.n] = 0;  // the offsets scan's sentinel
 }
 
 // One CTA per tile: move the tile's lists from the single-pass scratch into
@@ -743,7 +798,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_search_ell(Grid g, const int2* 
 // index, each tile particle's own staged index - and map every list entry to
 // its staged index.
 template <int T>
-__global__ void __launch_bounds__(T, 1152 / T) k_compact(Grid g, const int2* __restrict__ clin, Lin lin,
+__global__ void __launch_bounds__(T, 1152 / T) k_compact(const __grid_constant__ Grid g, const int2* __restrict__ clin, Lin lin,
                                                const int32_t* __restrict__ cellc,
                                                const float4* __restrict__ scr,
                                                const double* __restrict__ spos,
@@ -784,12 +839,19 @@ __global__ void __launch_bounds__(T, 1152 / T) k_compact(Grid g, const int2* __r
     }
     tmap[static_cast<int64_t>(blockIdx.x) * T + rank] = static_cast<uint8_t>(tid);
   }
-  if (tid < cnt) {
-    const int s = s0 + tid;
-    if (toff[tid + 1] > g.capacity) raise_flag(status_word, PHB_FLAG_CAPACITY);
-    if (ncnt[s] > g.ell)
-      search_overflow(g, clin, lin, cellc, scr, spos, list_radius(g, slam[s]), s, toff[tid],
-                                toff[tid + 1], idx);
+  if (tid < cnt && toff[tid + 1] > g.capacity) raise_flag(status_word, PHB_FLAG_CAPACITY);
+  // lists longer than their scratch rows: searched again by the warp (the
+  // shared arrays of the tile plan, not yet in use, hold its table)
+  {
+    const bool over = tid < cnt && ncnt[s0 + tid] > g.ell;
+    unsigned left = __ballot_sync(0xffffffffu, over);
+    for (; left != 0u; left &= left - 1u) {
+      const int p = (tid & ~31) + __ffs(left) - 1, s = s0 + p;
+      const int64_t to = toff[p] < g.capacity ? toff[p] : g.capacity;
+      search_overflow(g, lin, cellc, scr, spos, list_radius(g, slam[s]), s,
+                      base + (tid >> 5) * kWarpTable, g.capacity - to, idx + to);
+    }
+    __syncthreads();
   }
   tile_plan<T>(g, s0, cnt, cellc, slam, clin, ts, tarr);
   const bool staged = !ts.fallback;
@@ -1413,9 +1475,15 @@ cudaError_t build_neighbors_impl(const phb_plan* p, const double* pos, const dou
   note_launch();
   const Lin lin{lscr, lstart};
   int32_t* ell = region<int32_t>(p, ws, R_ELL);
-  // one lambda: cell-major, then particle-major for the lists it left;
-  // lambda varying: particle-major
-  const bool cell_major = p->lambda_max <= 1.01 * p->lambda_min;
+  // Which search (us of the search kernels).  One lambda: a warp per particle
+  // below kCellsMin (1,000 particles 15, 4,096: 18, 10,648: 29, 19,683: 43), from
+  // there on a warp per cell (37, 54, 40, 43; 262,144: 157), then a thread per
+  // particle for the lists it left.  Lambda varying: a warp per particle up to
+  // kWarpMax (10,007 particles 38, 60,000: 116, 130,000: 230), a thread per
+  // particle beyond (165, 181, 250; 260,000: 345 against 402).
+  constexpr int kCellsMin = 1 << 14, kWarpMax = 1 << 17;
+  const bool one_lambda = p->lambda_max <= 1.01 * p->lambda_min;
+  const bool cell_major = one_lambda && n >= kCellsMin;
   if (cell_major && (e = cudaMemsetAsync(ncnt, 0xff, static_cast<size_t>(n) * sizeof(int32_t), st)))
     return e;
   int tr = trace_begin(4, st);
@@ -1423,8 +1491,10 @@ cudaError_t build_neighbors_impl(const phb_plan* p, const double* pos, const dou
     k_search_cells<<<static_cast<unsigned>(ncells), 32, 0, st>>>(g, lin, spos, slam, ncnt, ell);
     note_launch();
   }
-  k_search_ell<<<blocks_for(n), kThreads, 0, st>>>(g, clin, lin, cellc, scr, spos, slam, ncnt, ell,
-                                                   cell_major);
+  if (cell_major || n > kWarpMax)
+    k_search_ell<<<blocks_for(n), kThreads, 0, st>>>(g, lin, cellc, scr, spos, slam, ncnt, ell, cell_major);
+  else
+    k_search_warp<<<blocks_for(n, 8), 128, 0, st>>>(g, lin, cellc, scr, spos, slam, ncnt, ell);
   trace_end(tr, st);
   note_launch();
   if ((e = scan_exclusive_i32_to_i64(ncnt, off, n + 1, bsum, st))) return e;
