@@ -25,7 +25,7 @@ enum Region {
   R_PERM,        // int32 [n]   slot -> caller index
   R_INV,         // int32 [n]   caller index -> slot
   R_CELL,        // int32 [nkeys+1] cell start (exclusive scan of counts)
-  R_CURSOR,      // int32 [nkeys]   scatter cursors
+  R_CURSOR,      // int32 [nkeys+1] scatter cursors
   R_SCAN,        // int64 [scan blocks] block sums
   R_SPOS,        // double [3][n] positions, slot order
   R_SLAM,        // double [n]    lambda, slot order

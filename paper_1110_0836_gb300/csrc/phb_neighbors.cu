@@ -16,7 +16,11 @@ constexpr int kOwnerCap = 8192;  // list entries of a tile mapped to their parti
 
 inline unsigned blocks_for(int64_t n, int t = kThreads) { return static_cast<unsigned>((n + t - 1) / t); }
 
-__global__ void k_keys(Grid g, const double* __restrict__ pos, const double* __restrict__ lam,
+// Cell keys and counts.  A particle without a finite position gets the key
+// after the last cell: it has no neighbours and is nobody's, so it must not
+// stand among a cell's candidates (157,000 of them in cell 0 made the search
+// of a blown-up 200,000-particle set 74 ms).
+__global__ void k_keys(Grid g, int32_t nkeys, const double* __restrict__ pos, const double* __restrict__ lam,
                        int32_t* __restrict__ keys, int32_t* __restrict__ counts,
                        int32_t* status_word) {
   const int n = g.n;
@@ -33,7 +37,7 @@ __global__ void k_keys(Grid g, const double* __restrict__ pos, const double* __r
   const double l = lam[i];
   if (!finite || !finite64(l)) raise_flag(status_word, PHB_FLAG_NONFINITE);
   if (!lambda_in_range(g, l)) raise_flag(status_word, PHB_FLAG_LAMBDA_RANGE);
-  const int32_t k = cell_key(g, c[0], c[1], c[2]);
+  const int32_t k = finite ? cell_key(g, c[0], c[1], c[2]) : nkeys;
   keys[i] = k;
   atomicAdd(&counts[k], 1);
 }
@@ -50,12 +54,12 @@ __global__ void k_scatter(int n, const int32_t* __restrict__ keys, const int32_t
 // Thread per particle: its rank among the particles of its cell is the number
 // of them with a smaller caller index (the cells' members come from the
 // atomic scatter in arbitrary order).  That is quadratic in a cell's members
-// (~12), so a cell of more than kBigCell - a clump, or the particles without a
-// finite position, which all go to cell 0 - is listed in one sweep of the
+// (~12), so a cell of more than kBigCell - a clump, or the key of the particles
+// without a finite position - is listed in one sweep of the
 // block that holds its first scattered member.
 constexpr int kBigCell = 2048;
 
-__global__ void __launch_bounds__(kThreads) k_rank_cells(int n, const int32_t* __restrict__ keys,
+__global__ void __launch_bounds__(kThreads) k_rank_cells(int n, int32_t nkeys, const int32_t* __restrict__ keys,
                                                          const int32_t* __restrict__ cell_start,
                                                          const int32_t* __restrict__ scattered,
                                                          int32_t* __restrict__ perm) {
@@ -64,7 +68,7 @@ __global__ void __launch_bounds__(kThreads) k_rank_cells(int n, const int32_t* _
   int32_t k = -1;
   if (i < n) {
     k = keys[i];
-    const int a = cell_start[k], b = cell_start[k + 1];
+    const int a = cell_start[k], b = k < nkeys ? cell_start[k + 1] : n;
     if (b - a <= kBigCell) {
       int rank = 0;
       for (int t = a; t < b; ++t) rank += scattered[t] < i ? 1 : 0;
@@ -153,7 +157,7 @@ __global__ void k_cell_lin(Grid g, const int32_t* __restrict__ cell_start, int2*
 // Screen records in linear cell order (z fastest; slot order inside a cell),
 // with the slot in w, plus four padding records: the cells of one (x, y) row
 // of a reach box are then one contiguous run.  lstart: exclusive scan of the
-// linear-order counts.
+// linear-order counts.  (Slots without a finite position have no record.)
 __global__ void k_fill_lin(Grid g, const int32_t* __restrict__ cellc, const int2* __restrict__ clin,
                            const int32_t* __restrict__ lstart, const float4* __restrict__ scr,
                            float4* __restrict__ lscr) {
@@ -163,7 +167,9 @@ __global__ void k_fill_lin(Grid g, const int32_t* __restrict__ cellc, const int2
   unpack_cell(cellc[s], cx, cy, cz);
   const int64_t k = (static_cast<int64_t>(cx) * g.ncell[1] + cy) * g.ncell[2] + cz;
   const float4 o = scr[s];
-  lscr[lstart[k] + (s - clin[k].x)] = make_float4(o.x, o.y, o.z, __int_as_float(s));
+  const int2 members = clin[k];
+  if (static_cast<unsigned>(s - members.x) < static_cast<unsigned>(members.y))
+    lscr[lstart[k] + (s - members.x)] = make_float4(o.x, o.y, o.z, __int_as_float(s));
   if (s < 4) lscr[g.n + s] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));  // batch padding
 }
 
@@ -868,7 +874,8 @@ __global__ void __launch_bounds__(T, 1152 / T) k_compact(const __grid_constant__
     if (tid < cnt) {
       const int s = s0 + tid;
       const int j = marked_index(tarr, box_index(g, ts, cellc[s]));
-      lself[s] = static_cast<uint16_t>(base[j] + (s - cstart[j]));
+      const int o = s - cstart[j];  // (a slot without a finite position is in no cell)
+      lself[s] = static_cast<uint16_t>(base[j] + (static_cast<unsigned>(o) < static_cast<unsigned>(base[j + 1] - base[j]) ? o : 0));
     }
   }
   // the tile's entries [e0, e1) as one flat range over the block (each
@@ -1452,16 +1459,17 @@ cudaError_t build_neighbors_impl(const phb_plan* p, const double* pos, const dou
   int32_t* misc = region<int32_t>(p, ws, R_MISC);
   cudaError_t e;
   // cell counts and scatter cursors are adjacent regions: one clear
-  const size_t clear = p->ws_off[R_CURSOR] + p->nkeys * sizeof(int32_t) - p->ws_off[R_CELL];
+  const int32_t nkeys = static_cast<int32_t>(p->nkeys);
+  const size_t clear = p->ws_off[R_CURSOR] + (p->nkeys + 1) * sizeof(int32_t) - p->ws_off[R_CELL];
   if ((e = cudaMemsetAsync(cell, 0, clear, st))) return e;
-  k_keys<<<blocks_for(n), kThreads, 0, st>>>(g, pos, lam, keys, cell, status_word);
+  k_keys<<<blocks_for(n), kThreads, 0, st>>>(g, nkeys, pos, lam, keys, cell, status_word);
   note_launch();
   if ((e = scan_exclusive_i32(cell, p->nkeys + 1, bsum, st))) return e;
   // the inverse-permutation region (written later by k_gather_pos) holds the
   // scattered order until the ranking puts it into ascending caller index
   k_scatter<<<blocks_for(n), kThreads, 0, st>>>(n, keys, cell, cursor, inv);
   note_launch();
-  k_rank_cells<<<blocks_for(n), kThreads, 0, st>>>(n, keys, cell, inv, perm);
+  k_rank_cells<<<blocks_for(n), kThreads, 0, st>>>(n, nkeys, keys, cell, inv, perm);
   note_launch();
   k_gather_pos<<<blocks_for(n), kThreads, 0, st>>>(g, perm, pos, lam, inv, spos, slam, scr, cellc);
   note_launch();

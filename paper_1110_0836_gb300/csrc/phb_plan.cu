@@ -317,7 +317,7 @@ extern "C" phb_status phb_plan_init(phb_plan* p) {
   sz[R_PERM] = n * 4;
   sz[R_INV] = n * 4;
   sz[R_CELL] = (nkeys + 1) * 4;
-  sz[R_CURSOR] = nkeys * 4;
+  sz[R_CURSOR] = (nkeys + 1) * 4;
   sz[R_SCAN] = (scan_blocks(std::max<int64_t>(nkeys + 1, n + 1)) + 1) * 8;
   sz[R_SPOS] = 3 * n * 8;
   sz[R_SLAM] = n * 8;
