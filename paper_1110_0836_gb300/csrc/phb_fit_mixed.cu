@@ -176,24 +176,27 @@ struct StagedSrc {
 // difference for the right-hand sides, so only the eight weighted basis
 // pairs the moments need are formed (the moments, in the packed pair layout,
 // are complete after pass A).
+// first: the first four list indices (pass A), loaded by the caller before the
+// staging's barrier; pass B's are requested before pass A's sums are parked.
 template <FitMode MODE, int T, class Src>
-__device__ __forceinline__ int accumulate(const Src& src, int64_t beg, int64_t end, float inv_l,
-                                          float inv_rf2, bool unweighted, float* park, int col,
-                                          float2 (&m2)[kNM2], float2 (&bB)[4][kNB2]) {
+__device__ __forceinline__ int accumulate(const Src& src, int64_t beg, int64_t end, const int (&first)[4],
+                                          float inv_l, float inv_rf2, bool unweighted, float* park,
+                                          int col, float2 (&m2)[kNM2], float2 (&bB)[4][kNB2]) {
   using G = Groups<MODE>;
   int cnt = 0;
 #pragma unroll
   for (int k = 0; k < kNM2; ++k) m2[k] = make_float2(0.f, 0.f);
+  int n1, n2, n3, n4;
   {
     float2 bA[G::NA][kNB2];
 #pragma unroll
     for (int f = 0; f < G::NA; ++f)
 #pragma unroll
       for (int j = 0; j < kNB2; ++j) bA[f][j] = make_float2(0.f, 0.f);
-    int n1 = beg < end ? src.index(beg) : 0;
-    int n2 = beg + 1 < end ? src.index(beg + 1) : 0;
-    int n3 = beg + 2 < end ? src.index(beg + 2) : 0;
-    int n4 = beg + 3 < end ? src.index(beg + 3) : 0;
+    n1 = first[0];
+    n2 = first[1];
+    n3 = first[2];
+    n4 = first[3];
     typename Src::RawA ra;
     if (Src::kPrefetch && beg < end) {
       ra = src.fetch_a(n1);
@@ -226,6 +229,10 @@ __device__ __forceinline__ int accumulate(const Src& src, int64_t beg, int64_t e
       mls_accum_rhs_basis2(qg2, wt * du[2], bA[G::NA - 2]);
       mls_accum_rhs_basis2(qg2, wt * du[3], bA[G::NA - 1]);
     }
+    n1 = beg < end ? src.index(beg) : 0;
+    n2 = beg + 1 < end ? src.index(beg + 1) : 0;
+    n3 = beg + 2 < end ? src.index(beg + 2) : 0;
+    n4 = beg + 3 < end ? src.index(beg + 3) : 0;
 #pragma unroll
     for (int f = 0; f < G::NA; ++f)
 #pragma unroll
@@ -235,10 +242,6 @@ __device__ __forceinline__ int accumulate(const Src& src, int64_t beg, int64_t e
   for (int f = 0; f < 4; ++f)
 #pragma unroll
     for (int j = 0; j < kNB2; ++j) bB[f][j] = make_float2(0.f, 0.f);
-  int n1 = beg < end ? src.index(beg) : 0;
-  int n2 = beg + 1 < end ? src.index(beg + 1) : 0;
-  int n3 = beg + 2 < end ? src.index(beg + 2) : 0;
-  int n4 = beg + 3 < end ? src.index(beg + 3) : 0;
   typename Src::RawB rb;
   if (Src::kPrefetch && beg < end) {
     rb = src.fetch_b(n1);
@@ -377,6 +380,17 @@ __device__ __forceinline__ void solve_fields(const float (&M)[kNT], const float 
   }
 }
 
+// v in FP64, on the integer pipe for normal numbers and zeros (a conversion
+// occupies the FP64 pipe for 17 SM cycles per warp).
+__device__ __forceinline__ double to_double(float v) {
+  const unsigned b = __float_as_uint(v), e = (b >> 23) & 0xffu;
+  if (e - 1u < 254u || (b << 1) == 0u) {
+    const unsigned mag = (b << 1) == 0u ? 0u : ((b & 0x7fffffffu) >> 3) + 0x38000000u;
+    return __hiloint2double(static_cast<int>(mag | (b & 0x80000000u)), static_cast<int>(b << 29));
+  }
+  return static_cast<double>(v);
+}
+
 // Outputs of one fitted slot from its parked derivative rows: fit status
 // and gradients / Hessians (derivative mode) or the MHD time derivatives.
 // Singular fits (too few neighbours) report zero derivatives.  No barrier.
@@ -420,16 +434,16 @@ __device__ __forceinline__ void write_outputs(const FitArgs& a, int s, bool sing
     float zeta = a.zeta ? static_cast<float>(a.zeta[src]) : 0.f;
     float eta = a.eta ? static_cast<float>(a.eta[src]) : 0.f;
     if (a.c_zeta_l != 0.0 || a.c_zeta_a != 0.0 || a.c_eta != 0.0)
-      mhd_laws(u, D, static_cast<float>(a.gamma), static_cast<float>(a.slam[s]),
+      mhd_laws(u, D, a.gamma32, static_cast<float>(a.slam[s]),
                static_cast<float>(a.c_zeta_l), static_cast<float>(a.c_zeta_a),
                static_cast<float>(a.c_eta), zeta, eta);
     float out[8];
-    mhd_rhs(u, D, static_cast<float>(a.gamma), zeta, eta, out);
+    mhd_rhs(u, D, a.gamma32, zeta, eta, out);
     bool finite = true;
 #pragma unroll
     for (int f = 0; f < 8; ++f) {
       finite &= isfinite(out[f]);
-      a.dudt[f * n + dst] = out[f];
+      a.dudt[f * n + dst] = to_double(out[f]);
     }
     if (!finite) raise_flag(a.status_word, PHB_FLAG_NONFINITE);
   }
@@ -455,33 +469,53 @@ struct FitShared {
   uint8_t fin[T];   // host-buffer corrector: the tile particle's fit is final here
 };
 
+constexpr int kStageBatch = 8;  // records per thread in flight
+
+// Slots of a thread's first batch of a tile's staged records (read before the
+// tile's count is known: entries past it are not used).
+template <int T>
+__device__ __forceinline__ void first_slots(const FitArgs& a, const int32_t* slots, int tid,
+                                            int (&first)[kStageBatch]) {
+#pragma unroll
+  for (int u = 0; u < kStageBatch; ++u) first[u] = tid + u * T < a.g.stage_cap ? slots[tid + u * T] : -1;
+}
+
 // Stage a tile's neighbourhood (count records, slots from the plan) in shared
 // memory: offsets and field differences relative to the tile's middle slot
 // sr, from the FP32 hi/lo records.  All T threads call it; no barrier inside.
 // Returns whether this thread staged an offset of a quarter box length or
 // more on a periodic axis (the tile's differences then need the wrap).
 template <int T>
-__device__ __forceinline__ bool stage_tile(const FitArgs& a, const Per32& P, const TileArgs& ta,
-                                           int tile, int sr, int count, float4* stage, int tid) {
+__device__ __forceinline__ bool stage_tile(const FitArgs& a, const Per32& P, const int32_t* slots,
+                                           const int (&first)[kStageBatch], int sr, int count,
+                                           float4* stage, int tid) {
   bool far = false;
   const float4* rec = reinterpret_cast<const float4*>(a.rec);
   // records relative to the tile's middle particle: the staged FP32 offsets
   // and field differences round to at most half the tile's extent
   const float4 rh = rec[6 * sr], rl = rec[6 * sr + 1];
   const float4 fh = rec[6 * sr + 2], fl = rec[6 * sr + 3], gh = rec[6 * sr + 4], gl = rec[6 * sr + 5];
-  const int32_t* slots = ta.tslot + static_cast<int64_t>(tile) * a.g.stage_cap;
-  // eight records per thread in flight: slots first, then all their loads
-  constexpr int kB = 8;
+  // eight records per thread in flight; their slots come a batch ahead (the
+  // first batch from the caller), so that no record waits for its slot
+  int ahead[kStageBatch];
+#pragma unroll
+  for (int u = 0; u < kStageBatch; ++u) ahead[u] = first[u];
+  constexpr int kB = kStageBatch;
   for (int l0 = tid; l0 < count; l0 += kB * T) {
     int sl[kB];
 #pragma unroll
-    for (int u = 0; u < kB; ++u) sl[u] = l0 + u * T < count ? slots[l0 + u * T] : -1;
+    for (int u = 0; u < kB; ++u) sl[u] = l0 + u * T < count ? ahead[u] : -1;
     float4 v[kB][6];
 #pragma unroll
     for (int u = 0; u < kB; ++u)
       if (sl[u] >= 0)
 #pragma unroll
         for (int k = 0; k < 6; ++k) v[u][k] = rec[6 * sl[u] + k];
+#pragma unroll
+    for (int u = 0; u < kB; ++u) {
+      const int l = l0 + (kB + u) * T;
+      ahead[u] = l < count ? slots[l] : -1;
+    }
 #pragma unroll
     for (int u = 0; u < kB; ++u) {
       if (sl[u] < 0) continue;
@@ -550,45 +584,60 @@ __device__ __forceinline__ void fit_tile(const FitArgs& a, const Per32& P, const
   const bool active = mine < cnt_tile;
   const int s = listed ? (active ? ta.list[s0 + mine] : 0) : s0 + mine;
 
-  // the neighbourhood planned by the neighbour build: one gather per staged record
+  // everything that needs no other load is requested here, before the
+  // staging and its barrier: the particle's list and scale, the tile's plan
+  // and the first slots to stage
+  const int32_t* slots = ta.tslot + static_cast<int64_t>(tile) * a.g.stage_cap;
+  int staged_first[kStageBatch];
+  if (!listed) first_slots<T>(a, slots, tid, staged_first);
   const int2 tp = listed ? make_int2(0, 1) : ta.tplan[tile];
+  int64_t beg = 0, end = 0;
+  double lam = 1.0;
+  int ls = 0;
+  if (active) {
+    lam = a.slam[s];
+    beg = a.off[s];
+    end = a.off[s + 1] < a.g.capacity ? a.off[s + 1] : a.g.capacity;
+    if (!listed) ls = ta.lself[s];
+  }
+  // the neighbourhood planned by the neighbour build: one gather per staged record
   const bool fb = tp.y != 0;
   if (!fb) {
-    const bool far = stage_tile<T>(a, P, ta, tile, s0 + (cnt_tile >> 1), tp.x, stage, tid);
+    const bool far = stage_tile<T>(a, P, slots, staged_first, s0 + (cnt_tile >> 1), tp.x, stage, tid);
     const bool wfar = __any_sync(0xffffffffu, far);
     if ((tid & 31) == 0) sh.wfar[tid >> 5] = wfar ? 1 : 0;
   } else if (tid == 0 && !listed) {
     atomicAdd(ta.fallback_count, 1);
   }
+  int first[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    first[k] = beg + k < end ? (fb ? a.idx[beg + k] : static_cast<int>(ta.lidx[beg + k])) : 0;
   __syncthreads();
 
   float2 m2[kNM2];
   float2 bB[4][kNB2];
   int cnt = 0;
   float inv_l = 1.f, inv_rf2 = 0.f;
-  int64_t beg = 0, end = 0;
   const bool unweighted = a.weight_kind == 1;
   if (active) {
     // the scales in FP32: two FP64 divisions per particle would queue on
     // GB300's narrow FP64 pipe whenever a CTA's threads start together
-    const float lamf = static_cast<float>(a.slam[s]);
-    const float rff = static_cast<float>(a.g.rf_factor) * lamf;
+    const float lamf = static_cast<float>(lam);
+    const float rff = a.rf32 * lamf;
     inv_l = 1.f / lamf;
     inv_rf2 = 1.f / (rff * rff);
-    beg = a.off[s];
-    end = a.off[s + 1] < a.g.capacity ? a.off[s + 1] : a.g.capacity;
     if (fb) {
       GlobalSrc src;
       src.rec = rec;
       src.idx = a.idx;
       for (int k = 0; k < 6; ++k) src.o[k] = rec[6 * s + k];
       src.P = P;
-      cnt = accumulate<MODE, T>(src, beg, end, inv_l, inv_rf2, unweighted, park, tid, m2, bB);
+      cnt = accumulate<MODE, T>(src, beg, end, first, inv_l, inv_rf2, unweighted, park, tid, m2, bB);
     } else {
       auto run = [&](auto src) {
         src.stage = stage;
         src.lidx = ta.lidx;
-        const int ls = ta.lself[s];
         src.me0 = stage[3 * ls];
         src.me1 = stage[3 * ls + 1];
         src.me2 = stage[3 * ls + 2];
@@ -596,7 +645,7 @@ __device__ __forceinline__ void fit_tile(const FitArgs& a, const Per32& P, const
           src.len[c] = P.len[c];
           src.inv_len[c] = P.inv_len[c];
         }
-        return accumulate<MODE, T>(src, beg, end, inv_l, inv_rf2, unweighted, park, tid, m2, bB);
+        return accumulate<MODE, T>(src, beg, end, first, inv_l, inv_rf2, unweighted, park, tid, m2, bB);
       };
       bool wrap = false;
       for (int w = 0; w < T / 32; ++w) wrap |= sh.wfar[w] != 0;
@@ -622,6 +671,9 @@ __device__ __forceinline__ void fit_tile(const FitArgs& a, const Per32& P, const
           mstash[(2 * k) * T + tid] = m2[k].x;
           mstash[(2 * k + 1) * T + tid] = m2[k].y;
         }
+      // the outputs' reads of the own record, on their way during the solves
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(rec + 6 * s + 2));
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(rec + 6 * s + 5));
       mls_assemble_p2(m2, M);
       const float minpiv = mls_cholesky<float>(M, invd);
       // conditioning estimate of the Jacobi-scaled matrix: n_b times the
@@ -783,7 +835,7 @@ __global__ void __launch_bounds__(T, 256 / T) k_fit_refine(const FitArgs a, cons
     const int s = a.rqueue[q];
     const float* st = a.rstash + q;
     const float lamf = static_cast<float>(a.slam[s]);
-    const float rff = static_cast<float>(a.g.rf_factor) * lamf;
+    const float rff = a.rf32 * lamf;
     const float inv_l = 1.f / lamf;
     const float inv_rf2 = 1.f / (rff * rff);
     const int64_t beg = a.off[s];
@@ -914,7 +966,12 @@ __global__ void __launch_bounds__(T, 2) k_gram_tc(const FitArgs a, const Per32 P
   const float4* rec = reinterpret_cast<const float4*>(a.rec);
   const int2 tp = ta.tplan[tile];
   const bool fb = tp.y != 0;
-  if (!fb) stage_tile<T>(a, P, ta, tile, s0 + (cnt_tile >> 1), tp.x, stage, tid);
+  if (!fb) {
+    const int32_t* slots = ta.tslot + static_cast<int64_t>(tile) * a.g.stage_cap;
+    int first[kStageBatch];
+    first_slots<T>(a, slots, tid, first);
+    stage_tile<T>(a, P, slots, first, s0 + (cnt_tile >> 1), tp.x, stage, tid);
+  }
   __syncthreads();
   const bool unweighted = a.weight_kind == 1;
   for (int p = 0; p < 32; ++p) {

@@ -408,6 +408,7 @@ struct FitArgs {
   const int64_t* off;          // [n+1]
   const int32_t* idx;          // [capacity]
   double gamma;
+  float gamma32, rf32;         // gamma and rf_factor in FP32
   int32_t weight_kind;
   float cond_threshold;
   const double* zeta;          // caller order (indexed through perm_in) or null

@@ -106,6 +106,8 @@ FitArgs fit_args(const phb_plan* plan, const phb_params* prm, void* ws, const in
   a.off = region<int64_t>(plan, ws, R_OFF);
   a.idx = region<int32_t>(plan, ws, R_IDX);
   a.gamma = prm->gamma;
+  a.gamma32 = static_cast<float>(prm->gamma);
+  a.rf32 = static_cast<float>(plan->rf_factor);
   a.weight_kind = prm->weight_kind;
   a.cond_threshold = static_cast<float>(prm->cond_threshold > 0 ? prm->cond_threshold : 3e4);
   a.zeta = prm->zeta;
