@@ -366,9 +366,11 @@ phb_status phb_pc_step_host(const phb_plan* plan, const phb_params* params, cons
  * the lists of the last build; dudt [8][n] and fit_status [n] (may be NULL)
  * are written at the listed caller indices only.  active: device int32
  * [n_active] caller indices (duplicates are evaluated once; an index outside
- * [0, n) is skipped and sets PHB_FLAG_BAD_INDEX).  The FP32-mixed path reads
- * neighbours through the unstaged (global-memory) form of the fused fit; the
- * FP64 path is the same kernel as the full evaluation.  Every particle's
+ * [0, n) is skipped and sets PHB_FLAG_BAD_INDEX).  The FP32-mixed path runs
+ * tile by tile as the full evaluation does when more than half of the
+ * particles are listed, and reads neighbours through the unstaged
+ * (global-memory) form of the fused fit otherwise; the FP64 path is the same
+ * kernel as the full evaluation.  Every particle's
  * pos, lambda and U are still read (neighbours of active particles). */
 phb_status phb_mhd_rhs_active(const phb_plan* plan, const phb_params* params, const double* pos,
                               const double* lambda, const double* U, const int32_t* active,

@@ -460,7 +460,16 @@ struct TileArgs {
   int32_t ntiles;
   const int32_t* list;      // active subset: slots (ascending), or null for all particles
   const int32_t* list_len;  // device count of the active subset
+  const int32_t* marks;     // exclusive scan of the active marks [n + 1] (launch of a CTA per tile), or null
 };
+
+// An active subset of more than half of the particles runs tile by tile like
+// the whole set, its tiles without active particles skipped: staged
+// neighbourhoods halve a fit's time (levels of a step are coherent in space, so
+// most tiles are all active or not at all; at random a half costs the same).
+__device__ __forceinline__ bool dense_subset(const TileArgs& ta, int n) {
+  return ta.marks != nullptr && 2 * static_cast<int64_t>(*ta.list_len) > n;
+}
 
 // Shared memory of one CTA besides the dynamic park/staging region.
 template <int T>
@@ -569,19 +578,25 @@ __device__ __forceinline__ void host_u_tile(const FitArgs& a, int s0, int cnt, c
 // T threads call it (it contains block barriers).  Threads are assigned to
 // the tile's particles in descending list length (map recorded by the
 // neighbour build) so that the lanes of a warp run loops of similar length.
-template <FitMode MODE, int T>
+template <FitMode MODE, int T, bool Subset>
 __device__ __forceinline__ void fit_tile(const FitArgs& a, const Per32& P, const TileArgs& ta,
                                          int tile, float* park, float4* stage, FitShared<T>& sh) {
   using G = Groups<MODE>;
   const int n = a.n;
   const int tid = threadIdx.x;
   const float4* rec = reinterpret_cast<const float4*>(a.rec);
-  // an active subset runs in chunks of T listed slots through the unstaged path
-  const bool listed = ta.list != nullptr;
+  // an active subset: as the whole set where it is dense, else in chunks of T
+  // listed slots through the unstaged path
+  const bool dense = Subset && dense_subset(ta, n);
+  const bool listed = Subset && !dense;
   const int s0 = tile * T;
   const int cnt_tile = min(T, (listed ? *ta.list_len : n) - s0);
   const int mine = listed ? tid : ta.tmap[static_cast<int64_t>(tile) * T + tid];
-  const bool active = mine < cnt_tile;
+  bool active = mine < cnt_tile;
+  if (dense) {
+    active = active && ta.marks[s0 + mine + 1] != ta.marks[s0 + mine];
+    if (!__syncthreads_or(active)) return;
+  }
   const int s = listed ? (active ? ta.list[s0 + mine] : 0) : s0 + mine;
 
   // everything that needs no other load is requested here, before the
@@ -791,7 +806,9 @@ __device__ __forceinline__ void fit_tile(const FitArgs& a, const Per32& P, const
   }
 }
 
-template <FitMode MODE, int T>
+// Subset: over the active subset ta.list (an instance of its own: the whole
+// set's does not pay for the choice of its path, 6 of 316 us).
+template <FitMode MODE, int T, bool Subset>
 __global__ void __launch_bounds__(T, 256 / T) k_fit_mixed(const FitArgs a, const Per32 P, const TileArgs ta) {
   using G = Groups<MODE>;
   // dynamic shared memory: [park A: NA*19 slots x T][staged records: stage_cap x 3 float4];
@@ -802,7 +819,7 @@ __global__ void __launch_bounds__(T, 256 / T) k_fit_mixed(const FitArgs a, const
   float4* stage = smem4 + (G::NA * kNB * T) / 4;
   // schedule 1: the block scheduler's dispatch order runs the tiles in
   // descending cost (longest first), without a loop over tiles in the kernel
-  fit_tile<MODE, T>(a, P, ta, ta.order ? ta.order[blockIdx.x] : static_cast<int>(blockIdx.x), park,
+  fit_tile<MODE, T, Subset>(a, P, ta, ta.order ? ta.order[blockIdx.x] : static_cast<int>(blockIdx.x), park,
                     stage, sh);
 }
 
@@ -1160,10 +1177,13 @@ cudaError_t launch_t(const FitArgs& a, const Per32& P, const TileArgs& ta, int64
   cudaError_t e;
   if (units == 0) return cudaGetLastError();
   {
-    cudaFuncSetAttribute(k_fit_mixed<MODE, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(smem));
+    auto kernel = k_fit_mixed<MODE, T, false>;
+    if constexpr (MODE == FitMode::kRHS) {  // (derivatives are never asked of a subset)
+      if (ta.list) kernel = k_fit_mixed<MODE, T, true>;
+    }
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     const int tr = trace_begin(1, st);
-    k_fit_mixed<MODE, T><<<tiles, T, smem, st>>>(a, P, ta);
+    kernel<<<tiles, T, smem, st>>>(a, P, ta);
     note_launch();
     trace_end(tr, st);
   }
@@ -1205,11 +1225,12 @@ cudaError_t launch_fit_mixed(const FitArgs& a, FitMode mode, const int2* tplan, 
                              const uint16_t* lself, const uint8_t* tmap, const uint16_t* lidx,
                              int32_t* fallback_count, const int32_t* order,
                              const int32_t* list, const int32_t* list_len, int64_t list_cap,
-                             cudaStream_t st) {
+                             const int32_t* marks, cudaStream_t st) {
   const Per32 P = make_per32(a.g);
   const TileArgs ta{tplan, tslot, lself, tmap, lidx, fallback_count,
                     (a.g.schedule == 1 && !list) ? order : nullptr,
-                    static_cast<int32_t>((a.n + a.g.tile - 1) / a.g.tile), list, list_len};
+                    static_cast<int32_t>((a.n + a.g.tile - 1) / a.g.tile), list, list_len,
+                    list_cap >= a.n ? marks : nullptr};
   if (mode == FitMode::kDerivs)
     return a.g.tile == 64 ? launch_t<FitMode::kDerivs, 64>(a, P, ta, list_cap, st)
                           : launch_t<FitMode::kDerivs, 128>(a, P, ta, list_cap, st);
@@ -1223,7 +1244,7 @@ cudaError_t launch_fit_tc(const FitArgs& a, const int2* tplan, const int32_t* ts
   if (a.g.tile != 128) return cudaErrorInvalidValue;
   const Per32 P = make_per32(a.g);
   const TileArgs ta{tplan, tslot, lself, tmap, lidx, nullptr, nullptr,
-                    static_cast<int32_t>((a.n + 127) / 128), nullptr, nullptr};
+                    static_cast<int32_t>((a.n + 127) / 128), nullptr, nullptr, nullptr};
   const size_t smem = size_t(a.g.stage_cap) * 3 * sizeof(float4) + 4 * kTcWarpFloats * sizeof(float);
   cudaFuncSetAttribute(k_gram_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        static_cast<int>(smem));

@@ -460,12 +460,14 @@ struct HostU {
 };
 
 // Fused FP32-mixed fit over all slots (list == null, staged tiles) or over
-// the slots list[0 .. *list_len) (at most list_cap; unstaged path).
+// the slots list[0 .. *list_len) (at most list_cap; unstaged path, or as the
+// whole set when they are many and list_cap reaches n; marks: the exclusive
+// scan of the listed slots' marks).
 cudaError_t launch_fit_mixed(const FitArgs& a, FitMode mode, const int2* tplan, const int32_t* tslot,
                              const uint16_t* lself, const uint8_t* tmap, const uint16_t* lidx,
                              int32_t* fallback_count, const int32_t* order,
                              const int32_t* list, const int32_t* list_len, int64_t list_cap,
-                             cudaStream_t st);
+                             const int32_t* marks, cudaStream_t st);
 // Tensor-core experiment: Gram matrices on mma.sync (3xTF32) into gram
 // [214][n], then the solve and right-hand side (tile 128 only).
 cudaError_t launch_fit_tc(const FitArgs& a, const int2* tplan, const int32_t* tslot,

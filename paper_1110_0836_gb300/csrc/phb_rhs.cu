@@ -168,7 +168,8 @@ cudaError_t run_fit(const phb_plan* plan, const phb_params* prm, void* ws, FitMo
   if ((e = launch_fit_mixed(a, mode, region<int2>(plan, ws, R_TPLAN), region<int32_t>(plan, ws, R_TSLOT),
                             region<uint16_t>(plan, ws, R_LSELF), tmap, region<uint16_t>(plan, ws, R_LIDX),
                             a.queue_len + 2,
-                            region<int32_t>(plan, ws, R_TORDER), list, list_len, list_cap, st)))
+                            region<int32_t>(plan, ws, R_TORDER), list, list_len, list_cap,
+                            list ? region<int32_t>(plan, ws, R_AFLAG) : nullptr, st)))
     return e;
   return launch_fit_fp64(a, mode, a.queue, a.queue_len, tmap, st, true);
 }
@@ -240,7 +241,8 @@ extern "C" phb_status phb_mhd_rhs_active(const phb_plan* plan, const phb_params*
   k_list_active<<<static_cast<unsigned>((n + 1 + kThreads - 1) / kThreads), kThreads, 0, st>>>(
       n, mark, list, list_len);
   note_launch();
-  const int64_t cap = n_active < n ? n_active : n;
+  // half of the particles or more may run tile by tile (see dense_subset)
+  const int64_t cap = 2 * n_active > n ? n : n_active;
   e = run_fit(plan, prm, ws, FitMode::kRHS, region<int32_t>(plan, ws, R_PERM), dudt, nullptr,
               nullptr, fit_status, status_word, st, list, list_len, cap);
   return launch_status(e);
