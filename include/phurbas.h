@@ -164,7 +164,7 @@ typedef struct {
   int32_t nbrick[3];     /* 4x4x4-cell bricks per axis */
   int32_t hilbert_bits;  /* bricks are ordered along a 3-D Hilbert curve of this order */
   int32_t ntiles;        /* ceil(n / tile) */
-  int64_t nkeys;         /* cell-key space: bricks * 64 */
+  int64_t nkeys;         /* cell-key space: bricks (of the grid, or of the Hilbert cube) * 64 */
   double screen_margin;  /* absolute distance margin of the FP32 neighbour screen */
   size_t ws_bytes;       /* workspace bytes needed for every operation */
   size_t ws_off[48];     /* byte offsets of the workspace regions (internal) */

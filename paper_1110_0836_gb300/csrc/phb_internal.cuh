@@ -52,6 +52,8 @@ enum Region {
   R_RQUEUE,      // int32 [n]    slots of refined tiles' fits, queued for the corrected step
   R_RSTASH,      // float [80 + 8*19][n] per queued fit (queue order): its moments in the
                  //   packed pair layout, then the 19 first-solve coefficients of each field
+  R_BBITS,       // uint32 [brick_words] bricks of the Hilbert cube that the grid has (compact keys)
+  R_BBEFORE,     // int32 [brick_words+1] bricks before each of those words
   R_DIAG,        // double [3][kDiagBlocks] block partial sums of the mode-amplitude diagnostic
   R_PC_F0,       // double [8][n] F(Y^n) (slot order)        -- PC step
   R_PC_F1,       // double [8][n] F(Y^p) (slot order)        -- PC step
@@ -98,6 +100,10 @@ struct Grid {
 };
 
 Grid make_grid(const phb_plan* p);
+
+// Words of the bricks' bitmap when the plan's keys count only the grid's
+// bricks, else 0.
+int64_t brick_words(const phb_plan* p);
 
 // Rows (list entries) of the adjoint's term buffer: all list entries of sets up
 // to 2^17 particles (2^23 rows at most), else 28 per particle - the entries
@@ -257,12 +263,22 @@ __host__ __device__ inline uint32_t hilbert3(uint32_t x, uint32_t y, uint32_t z,
   return h;
 }
 
+// Ranks of the grid's bricks along the Hilbert curve, where the curve's cube
+// holds many more bricks than the grid (elongated boxes): a bit per brick of
+// the cube and the bricks before each word.  Null: the curve index itself.
+struct Bricks {
+  const uint32_t* bits;
+  const int32_t* before;
+};
+
 // Cell key: 4x4x4-cell bricks ordered along the Hilbert curve, Morton order of
 // the 64 cells inside a brick.  Cells that are close in space get close keys,
 // so a run of consecutive particles covers a compact region.
-__device__ __forceinline__ int32_t cell_key(const Grid& g, int cx, int cy, int cz) {
-  const uint32_t hb = hilbert3(static_cast<uint32_t>(cx >> 2), static_cast<uint32_t>(cy >> 2),
-                               static_cast<uint32_t>(cz >> 2), g.hbits);
+__device__ __forceinline__ int32_t cell_key(const Grid& g, const Bricks& br, int cx, int cy, int cz) {
+  uint32_t hb = hilbert3(static_cast<uint32_t>(cx >> 2), static_cast<uint32_t>(cy >> 2),
+                         static_cast<uint32_t>(cz >> 2), g.hbits);
+  if (br.bits)
+    hb = static_cast<uint32_t>(br.before[hb >> 5]) + __popc(br.bits[hb >> 5] & ((1u << (hb & 31u)) - 1u));
   int x = cx & 3, y = cy & 3, z = cz & 3;
   int m = (x & 1) | ((y & 1) << 1) | ((z & 1) << 2) | ((x & 2) << 2) | ((y & 2) << 3) | ((z & 2) << 4);
   return static_cast<int32_t>(hb * 64u + static_cast<uint32_t>(m));

@@ -16,11 +16,27 @@ constexpr int kOwnerCap = 8192;  // list entries of a tile mapped to their parti
 
 inline unsigned blocks_for(int64_t n, int t = kThreads) { return static_cast<unsigned>((n + t - 1) / t); }
 
+// The grid's bricks in the bitmap of the Hilbert cube, and the bricks per word
+// (whose exclusive scan is Bricks::before).
+__global__ void k_brick_mark(Grid g, uint32_t* __restrict__ bits) {
+  const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int nz = g.nbrick[2], ny = g.nbrick[1];
+  if (k >= static_cast<int64_t>(g.nbrick[0]) * ny * nz) return;
+  const uint32_t h = hilbert3(static_cast<uint32_t>(k / (static_cast<int64_t>(ny) * nz)),
+                              static_cast<uint32_t>(k / nz % ny), static_cast<uint32_t>(k % nz), g.hbits);
+  atomicOr(&bits[h >> 5], 1u << (h & 31u));
+}
+
+__global__ void k_brick_count(int64_t words, const uint32_t* __restrict__ bits, int32_t* __restrict__ before) {
+  const int64_t w = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (w <= words) before[w] = w < words ? __popc(bits[w]) : 0;
+}
+
 // Cell keys and counts.  A particle without a finite position gets the key
 // after the last cell: it has no neighbours and is nobody's, so it must not
 // stand among a cell's candidates (157,000 of them in cell 0 made the search
 // of a blown-up 200,000-particle set 74 ms).
-__global__ void k_keys(Grid g, int32_t nkeys, const double* __restrict__ pos, const double* __restrict__ lam,
+__global__ void k_keys(Grid g, Bricks br, int32_t nkeys, const double* __restrict__ pos, const double* __restrict__ lam,
                        int32_t* __restrict__ keys, int32_t* __restrict__ counts,
                        int32_t* status_word) {
   const int n = g.n;
@@ -37,7 +53,7 @@ __global__ void k_keys(Grid g, int32_t nkeys, const double* __restrict__ pos, co
   const double l = lam[i];
   if (!finite || !finite64(l)) raise_flag(status_word, PHB_FLAG_NONFINITE);
   if (!lambda_in_range(g, l)) raise_flag(status_word, PHB_FLAG_LAMBDA_RANGE);
-  const int32_t k = finite ? cell_key(g, c[0], c[1], c[2]) : nkeys;
+  const int32_t k = finite ? cell_key(g, br, c[0], c[1], c[2]) : nkeys;
   keys[i] = k;
   atomicAdd(&counts[k], 1);
 }
@@ -136,7 +152,7 @@ __global__ void k_gather_pos(Grid g, const int32_t* __restrict__ perm, const dou
 // (first slot, count) of every cell by linear index, for the tile planner and
 // the search; the counts also go to lcnt[k] (lcnt[total] = 0), whose
 // exclusive scan places the cells in linear order for the run search.
-__global__ void k_cell_lin(Grid g, const int32_t* __restrict__ cell_start, int2* __restrict__ clin,
+__global__ void k_cell_lin(Grid g, Bricks br, const int32_t* __restrict__ cell_start, int2* __restrict__ clin,
                            int32_t* __restrict__ lcnt, int32_t* __restrict__ misc) {
   const int64_t total = static_cast<int64_t>(g.ncell[0]) * g.ncell[1] * g.ncell[2];
   const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -148,7 +164,7 @@ __global__ void k_cell_lin(Grid g, const int32_t* __restrict__ cell_start, int2*
   const int cz = static_cast<int>(k % g.ncell[2]);
   const int cy = static_cast<int>((k / g.ncell[2]) % g.ncell[1]);
   const int cx = static_cast<int>(k / (static_cast<int64_t>(g.ncell[2]) * g.ncell[1]));
-  const int32_t key = cell_key(g, cx, cy, cz);
+  const int32_t key = cell_key(g, br, cx, cy, cz);
   const int a = cell_start[key];
   clin[k] = make_int2(a, cell_start[key + 1] - a);
   lcnt[k] = cell_start[key + 1] - a;
@@ -1462,7 +1478,19 @@ cudaError_t build_neighbors_impl(const phb_plan* p, const double* pos, const dou
   const int32_t nkeys = static_cast<int32_t>(p->nkeys);
   const size_t clear = p->ws_off[R_CURSOR] + (p->nkeys + 1) * sizeof(int32_t) - p->ws_off[R_CELL];
   if ((e = cudaMemsetAsync(cell, 0, clear, st))) return e;
-  k_keys<<<blocks_for(n), kThreads, 0, st>>>(g, nkeys, pos, lam, keys, cell, status_word);
+  Bricks br{nullptr, nullptr};
+  if (const int64_t words = brick_words(p); words > 0) {
+    uint32_t* bits = region<uint32_t>(p, ws, R_BBITS);
+    int32_t* before = region<int32_t>(p, ws, R_BBEFORE);
+    if ((e = cudaMemsetAsync(bits, 0, words * sizeof(uint32_t), st))) return e;
+    k_brick_mark<<<blocks_for(p->nkeys / 64), kThreads, 0, st>>>(g, bits);
+    note_launch();
+    k_brick_count<<<blocks_for(words + 1), kThreads, 0, st>>>(words, bits, before);
+    note_launch();
+    if ((e = scan_exclusive_i32(before, words + 1, bsum, st))) return e;
+    br = Bricks{bits, before};
+  }
+  k_keys<<<blocks_for(n), kThreads, 0, st>>>(g, br, nkeys, pos, lam, keys, cell, status_word);
   note_launch();
   if ((e = scan_exclusive_i32(cell, p->nkeys + 1, bsum, st))) return e;
   // the inverse-permutation region (written later by k_gather_pos) holds the
@@ -1476,7 +1504,7 @@ cudaError_t build_neighbors_impl(const phb_plan* p, const double* pos, const dou
   const int64_t ncells = int64_t(p->ncell[0]) * p->ncell[1] * p->ncell[2];
   int32_t* lstart = region<int32_t>(p, ws, R_LSTART);
   float4* lscr = region<float4>(p, ws, R_LSCR);
-  k_cell_lin<<<blocks_for(ncells + 1), kThreads, 0, st>>>(g, cell, clin, lstart, misc);
+  k_cell_lin<<<blocks_for(ncells + 1), kThreads, 0, st>>>(g, br, cell, clin, lstart, misc);
   note_launch();
   if ((e = scan_exclusive_i32(lstart, ncells + 1, bsum, st))) return e;
   k_fill_lin<<<blocks_for(n), kThreads, 0, st>>>(g, cellc, clin, lstart, scr, lscr);

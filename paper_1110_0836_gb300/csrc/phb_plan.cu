@@ -46,6 +46,17 @@ Grid make_grid(const phb_plan* p) {
   return g;
 }
 
+int64_t brick_words(const phb_plan* p) {
+  // A build clears, counts and scans all keys.  Builds of 200,000 particles in
+  // boxes of 15, 29, 58, 116 and 216 x 2 x 2 bricks (cubes of 2^12 to 2^24
+  // bricks): 2,675, 1,014, 490, 1,319 and 8,555 us with the cube's keys; 2,680,
+  // 1,005, 389, 301 and 309 us with ranks, whose six launches take 10 us.  An
+  // 8 x 1 x 1 tube's key arrays shrink from 134 MB to 0.5 MB.
+  const int64_t cube = int64_t(1) << (3 * p->hilbert_bits);
+  const int64_t bricks = int64_t(p->nbrick[0]) * p->nbrick[1] * p->nbrick[2];
+  return cube >= (int64_t(1) << 15) && 4 * bricks <= cube ? cube / 32 : 0;
+}
+
 int64_t adjoint_rows(const phb_plan* p) {
   const int64_t all = std::max<int64_t>(p->nbr_capacity, 1) + p->n, some = 28 * p->n;
   return p->n > int64_t(1) << 17 ? some : std::max(some, std::min<int64_t>(all, int64_t(1) << 23));
@@ -287,8 +298,9 @@ extern "C" phb_status phb_plan_init(phb_plan* p) {
   int hb = 0;
   while ((1 << hb) < maxb) ++hb;
   p->hilbert_bits = hb;
-  const int64_t nkeys = (int64_t(1) << (3 * hb)) * 64;
+  int64_t nkeys = (int64_t(1) << (3 * hb)) * 64;
   if (nkeys >= (int64_t(1) << 31) - 2) return PHB_ERR_INVALID_ARG;
+  if (brick_words(p) > 0) nkeys = int64_t(64) * p->nbrick[0] * p->nbrick[1] * p->nbrick[2];
   p->nkeys = nkeys;
   if (p->tile == 0) p->tile = 128;
   if (p->tile != 64 && p->tile != 128) return PHB_ERR_INVALID_ARG;
@@ -318,7 +330,8 @@ extern "C" phb_status phb_plan_init(phb_plan* p) {
   sz[R_INV] = n * 4;
   sz[R_CELL] = (nkeys + 1) * 4;
   sz[R_CURSOR] = (nkeys + 1) * 4;
-  sz[R_SCAN] = (scan_blocks(std::max<int64_t>(nkeys + 1, n + 1)) + 1) * 8;
+  const int64_t words = brick_words(p);
+  sz[R_SCAN] = (scan_blocks(std::max({nkeys + 1, n + 1, words + 1})) + 1) * 8;
   sz[R_SPOS] = 3 * n * 8;
   sz[R_SLAM] = n * 8;
   sz[R_SU] = 8 * n * 8;
@@ -343,6 +356,8 @@ extern "C" phb_status phb_plan_init(phb_plan* p) {
   sz[R_QUEUE] = (n + 64) * 4;  // also the export's n+1 counts
   sz[R_RQUEUE] = size_t(n) * 4;
   sz[R_RSTASH] = size_t(80 + kNF * 19) * n * 4;
+  sz[R_BBITS] = size_t(words) * 4;
+  sz[R_BBEFORE] = size_t(words > 0 ? words + 1 : 0) * 4;
   sz[R_DIAG] = size_t(3) * kDiagBlocks * 8;
   size_t off = 0;
   for (int r = R_MISC; r <= R_DIAG; ++r) {

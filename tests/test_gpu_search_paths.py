@@ -85,3 +85,21 @@ def test_crowded_cells_and_lost_particles():
     assert np.array_equal(np.sort(perm), np.arange(n))
     # the crowd shares one cell: its storage order is by caller index
     assert (np.diff(at[np.sort(crowd)]) > 0).all()
+
+
+@pytest.mark.parametrize("lengths,periodic", [((40.0, 1.0, 1.0), (1, 1, 1)), ((1.0, 1.0, 23.0), (0, 0, 0)),
+                                              ((1.0, 34.5, 0.9), (0, 1, 0))])
+def test_keys_of_the_grids_own_bricks(lengths, periodic):
+    """Boxes whose Hilbert cube holds many more bricks than the grid, on both
+    sides of the line from which keys are ranks of the grid's bricks: wrong
+    ranks would merge or lose cells."""
+    phb = need_gpu()
+    rng = np.random.default_rng(11)
+    n, L = 20_003, np.array(lengths)
+    w = workloads.Workload("long", -0.3 * L, 0.7 * L, np.array(periodic, np.int32),
+                           (rng.uniform(-0.3, 0.7, (n, 3)) * L).T.copy(), rng.uniform(0.06, 0.09, n),
+                           workloads.configs.background(n), 5.0 / 3.0)
+    plan = phb.Plan.for_workload(w)
+    cube, bricks = 8 ** plan.c.hilbert_bits, int(np.prod(list(plan.c.nbrick)))
+    assert plan.c.nkeys == 64 * (bricks if cube >= 2 ** 15 and 4 * bricks <= cube else cube)
+    check(w, sets(phb, w), sample(n, 500, seed=6))
