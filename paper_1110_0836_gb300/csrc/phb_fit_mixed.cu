@@ -67,6 +67,17 @@ struct Groups {
   }
 };
 
+// 32 bytes of a record (float4 pair k of 0, 1, 2; records are 96 bytes, 32-byte
+// aligned) in one load.  A gather's lanes read different records, so each of
+// its instructions costs the L1 a lookup per lane whatever its width.  Against
+// two 16-byte loads: 1M-tube step 8.00 -> 7.79 ms (corrected step and staging),
+// 64^3 step 0.991 -> 0.978 ms (staging), 8M-layer step 69.8 -> 68.8 ms.
+__device__ __forceinline__ void load_pair(const float4* rec, int t, int k, float4& a, float4& b) {
+  asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+      : "l"(rec + 6 * static_cast<int64_t>(t) + 2 * k));
+}
+
 // Neighbour data from the FP32 hi/lo records in global memory.
 // du (pass A) = (rho, sigma, Vx, Vy) differences; (pass B) = (Vz, Bx, By, Bz).
 // fetch_* issues a neighbour's loads, decode_* turns them into offsets and
@@ -83,11 +94,19 @@ struct GlobalSrc {
   using RawA = Raw;
   using RawB = Raw;
   __device__ __forceinline__ int index(int64_t e) const { return idx[e]; }
+  // the aligned pair that holds entry e (the list region is a multiple of 256 bytes)
+  __device__ __forceinline__ int2 index2(int64_t e) const { return reinterpret_cast<const int2*>(idx)[e >> 1]; }
   __device__ __forceinline__ Raw fetch_a(int t) const {
-    return Raw{rec[6 * t], rec[6 * t + 1], rec[6 * t + 2], rec[6 * t + 3]};
+    Raw r;
+    load_pair(rec, t, 0, r.p0, r.p1);
+    load_pair(rec, t, 1, r.h, r.l);
+    return r;
   }
   __device__ __forceinline__ Raw fetch_b(int t) const {
-    return Raw{rec[6 * t], rec[6 * t + 1], rec[6 * t + 4], rec[6 * t + 5]};
+    Raw r;
+    load_pair(rec, t, 0, r.p0, r.p1);
+    load_pair(rec, t, 2, r.h, r.l);
+    return r;
   }
   __device__ __forceinline__ void offs(const Raw& r, float& dx, float& dy, float& dz) const {
     dx = mi_diff32(r.p0.x, r.p1.x, o[0].x, o[1].x, P.len_h[0], P.len_l[0], P.inv_len[0]);
@@ -271,13 +290,54 @@ __device__ __forceinline__ int accumulate(const Src& src, int64_t beg, int64_t e
   return cnt;
 }
 
+// A list's entry after the one in use, loaded two to four entries before it
+// is used: one entry at a time, or the aligned pair of two.  Inside a tile the
+// staging leaves 28 KB of L1, less than the 32-byte sectors that 256 threads'
+// lists and records want to keep: pairs halve the lists' lookups, and a sector
+// lost before its next use costs half as much (8M-layer step 68.8 -> 65.5 ms;
+// groups of four 66.1).  The queue's kernel has 90 KB of L1 and no register
+// to spare (1M-tube step 7.78 ms with single entries, 8.10 with pairs).
+template <bool Pairs>
+struct Ahead {
+  int i2, i3;
+  template <class Src>
+  __device__ __forceinline__ Ahead(const Src& src, int64_t beg, int64_t end) {
+    i2 = beg + 1 < end ? src.index(beg + 1) : 0;
+    i3 = beg + 2 < end ? src.index(beg + 2) : 0;
+  }
+  __device__ __forceinline__ int at(int64_t) const { return i2; }
+  template <class Src>
+  __device__ __forceinline__ void advance(const Src& src, int64_t e, int64_t end) {
+    i2 = i3;
+    if (e + 3 < end) i3 = src.index(e + 3);
+  }
+};
+
+template <>
+struct Ahead<true> {
+  int2 p2, p3;  // the pair of entry e + 1 and the one after it
+  template <class Src>
+  __device__ __forceinline__ Ahead(const Src& src, int64_t beg, int64_t end) {
+    const int64_t second = ((beg + 1) | 1) + 1;
+    p2 = beg + 1 < end ? src.index2(beg + 1) : make_int2(0, 0);
+    p3 = second < end ? src.index2(second) : make_int2(0, 0);
+  }
+  __device__ __forceinline__ int at(int64_t e) const { return (e & 1) ? p2.x : p2.y; }
+  template <class Src>
+  __device__ __forceinline__ void advance(const Src& src, int64_t e, int64_t end) {
+    if (e & 1) return;
+    p2 = p3;
+    if (e + 4 < end) p3 = src.index2(e + 4);
+  }
+};
+
 // One corrected semi-normal-equations pass for the fields of slots
 // [k0, k0 + NFG): c0 (all 19 coefficients of each, from the fit's column cg
 // of the stash, stride cs) in registers, residuals r_j = du_j - p(q_j).c0
 // recomputed from the global records (RawA = RawB there),
 // acc_k = sum_j w_j p(q_j) r_j.  B selects the record half (false: rho,
 // sigma, Vx, Vy; true: Vz, Bx, By, Bz); du0 is the first du component used.
-template <int NFG, bool B, class Src>
+template <int NFG, bool B, bool Pairs, class Src>
 __device__ __forceinline__ void csne_pass(const Src& src, int64_t beg, int64_t end, float inv_l,
                                           float inv_rf2, bool unweighted, const float* cg,
                                           int64_t cs, int k0, int du0, float2 (&acc)[NFG][kNB2]) {
@@ -295,14 +355,15 @@ __device__ __forceinline__ void csne_pass(const Src& src, int64_t beg, int64_t e
   // index loaded two neighbours before that (so that the record's load does
   // not wait on its index's)
   typename Src::RawB nxt;
-  int i2 = beg + 1 < end ? src.index(beg + 1) : 0;
-  int i3 = beg + 2 < end ? src.index(beg + 2) : 0;
+  Ahead<Pairs> next(src, beg, end);
   if (beg < end) nxt = B ? src.fetch_b(src.index(beg)) : src.fetch_a(src.index(beg));
   for (int64_t e = beg; e < end; ++e) {
     const typename Src::RawB cur = nxt;
-    if (e + 1 < end) nxt = B ? src.fetch_b(i2) : src.fetch_a(i2);
-    i2 = i3;
-    if (e + 3 < end) i3 = src.index(e + 3);
+    if (e + 1 < end) {
+      const int t = next.at(e);
+      nxt = B ? src.fetch_b(t) : src.fetch_a(t);
+    }
+    next.advance(src, e, end);
     float dx, dy, dz, du[4];
     if (B) src.decode_b(cur, dx, dy, dz, du);
     else src.decode_a(cur, dx, dy, dz, du);
@@ -319,6 +380,14 @@ __device__ __forceinline__ void csne_pass(const Src& src, int64_t beg, int64_t e
   }
 }
 
+
+// Requests entries [beg, end) of the neighbour list into L2.  The fused fit
+// reads its tile's 16-bit indices, so a refined tile's lists come from DRAM:
+// asked for before the first solves (8M-layer step 71.4 -> 69.8 ms).
+__device__ __forceinline__ void prefetch_list(const int32_t* idx, int64_t beg, int64_t end) {
+  for (int64_t e = beg; e < end; e += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(idx + e));
+  if (beg < end) asm volatile("prefetch.global.L2 [%0];" ::"l"(idx + end - 1));
+}
 
 // Linear and quadratic coefficients b[10..18] -> derivatives in the first
 // nine rows of the parked column (gradient, then the packed Hessian).
@@ -519,7 +588,7 @@ __device__ __forceinline__ bool stage_tile(const FitArgs& a, const Per32& P, con
     for (int u = 0; u < kB; ++u)
       if (sl[u] >= 0)
 #pragma unroll
-        for (int k = 0; k < 6; ++k) v[u][k] = rec[6 * sl[u] + k];
+        for (int k = 0; k < 3; ++k) load_pair(rec, sl[u], k, v[u][2 * k], v[u][2 * k + 1]);
 #pragma unroll
     for (int u = 0; u < kB; ++u) {
       const int l = l0 + (kB + u) * T;
@@ -706,6 +775,7 @@ __device__ __forceinline__ void fit_tile(const FitArgs& a, const Per32& P, const
   // one decision per tile keeps the CTA's control flow uniform
   const bool refine = may_refine && __syncthreads_or(need);
   if (refine && tid == 0) atomicAdd(a.refined_tiles, 1);
+  if (refine && !a.refine_queued && !fb) prefetch_list(a.idx, beg, end);
   const bool solve = !singular && !routed;
   const float il = inv_l, il2 = inv_l * inv_l;
   if (solve && !refine) {
@@ -764,7 +834,7 @@ __device__ __forceinline__ void fit_tile(const FitArgs& a, const Per32& P, const
     src.P = P;
     {
       float2 acc[G::NA][kNB2];
-      csne_pass<G::NA, false>(src, beg, end, inv_l, inv_rf2, unweighted, park + tid, T, 0,
+      csne_pass<G::NA, false, true>(src, beg, end, inv_l, inv_rf2, unweighted, park + tid, T, 0,
                               4 - G::NA, acc);
 #pragma unroll
       for (int f = 0; f < G::NA; ++f)
@@ -773,7 +843,7 @@ __device__ __forceinline__ void fit_tile(const FitArgs& a, const Per32& P, const
     }
     {
       float2 acc[4][kNB2];
-      csne_pass<4, true>(src, beg, end, inv_l, inv_rf2, unweighted, park + tid, T, G::NA, 0, acc);
+      csne_pass<4, true, true>(src, beg, end, inv_l, inv_rf2, unweighted, park + tid, T, G::NA, 0, acc);
 #pragma unroll
       for (int f = 0; f < 4; ++f)
 #pragma unroll
@@ -866,7 +936,7 @@ __global__ void __launch_bounds__(T, 256 / T) k_fit_refine(const FitArgs a, cons
     src.P = P;
     {
       float2 acc[G::NA][kNB2];
-      csne_pass<G::NA, false>(src, beg, end, inv_l, inv_rf2, unweighted, st + kNM * n, n, 0,
+      csne_pass<G::NA, false, false>(src, beg, end, inv_l, inv_rf2, unweighted, st + kNM * n, n, 0,
                               4 - G::NA, acc);
 #pragma unroll
       for (int f = 0; f < G::NA; ++f)
@@ -877,7 +947,7 @@ __global__ void __launch_bounds__(T, 256 / T) k_fit_refine(const FitArgs a, cons
       src.o[4] = rec[6 * s + 4];
       src.o[5] = rec[6 * s + 5];
       float2 acc[4][kNB2];
-      csne_pass<4, true>(src, beg, end, inv_l, inv_rf2, unweighted, st + kNM * n, n, G::NA, 0, acc);
+      csne_pass<4, true, false>(src, beg, end, inv_l, inv_rf2, unweighted, st + kNM * n, n, G::NA, 0, acc);
 #pragma unroll
       for (int f = 0; f < 4; ++f)
 #pragma unroll
