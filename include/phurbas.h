@@ -128,10 +128,9 @@ typedef struct {
    * -1 never refines. */
   int32_t refine;
   /* Where the corrected step of refined tiles runs: 0 = by the set (a second
-   * kernel over a queue of the refined tiles' fits when n x 96 B of FP32
-   * records fit in the device's L2 and lambda varies - sets of one
-   * resolution rarely refine and skip that launch - inside the tile
-   * otherwise), 1 = the queue, 2 = inside the tile (other values: as 0).
+   * kernel over a queue of the refined tiles' fits for fewer than 65,536 fits
+   * of varying lambda - sets of one resolution rarely refine and skip that
+   * launch - inside the tile otherwise), 1 = the queue, 2 = inside the tile (other values: as 0).
    * Same results either way. */
   int32_t refine_schedule;
   double refine_kappa;

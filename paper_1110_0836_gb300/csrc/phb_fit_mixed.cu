@@ -28,11 +28,11 @@
 // r_j = (U_j - U_i) - p(q_j).c0 recomputed from the records, and the same
 // factor (re-formed from the kept moments) solves for the correction.  The
 // error then follows cond(A) = cond(M_s)^(1/2) instead of cond(M_s).  The
-// decision is per tile (a per-fit rule leaves fits above the bar).  Where the
-// set's FP32 records fit in L2, a refined tile queues its fits with their
-// moments and c0 for k_fit_refine, which streams through the queue without
-// the tile's barriers; larger sets take the step inside the tile, while its
-// neighbourhood is still in L2.
+// decision is per tile (a per-fit rule leaves fits above the bar).  In small
+// sets of varying lambda a refined tile queues its fits with their moments and
+// c0 for k_fit_refine, which streams through the queue without the tile's
+// barriers; other sets take the step inside the tile, while its neighbourhood
+// is still in L2.
 #include "phb_internal.cuh"
 #include "mls_gen.cuh"
 #include "phb_mhd.cuh"
@@ -783,7 +783,7 @@ __device__ __forceinline__ void fit_tile(const FitArgs& a, const Per32& P, const
         M, invd, [&](int k, int j) { return park[(k * kNB + j) * T + tid]; },
         [&](int k, const float(&b)[kNB]) { park_derivs<T>(park + (k * kNB) * T + tid, b, il, il2); });
   }
-  // A refined tile of a set whose records fit in L2 hands its solved fits to
+  // A refined tile of a small set (FitArgs::refine_queued) hands its solved fits to
   // k_fit_refine: one queue position per fit (one atomic per warp), its
   // moments and the first solve's 19 coefficients of every field into the
   // queue's stash.  (Before the in-tile step below, so that the factor is
@@ -812,7 +812,7 @@ __device__ __forceinline__ void fit_tile(const FitArgs& a, const Per32& P, const
   }
   if (solve && refine && !a.refine_queued) {
     // Otherwise the corrected step here, while the tile's neighbourhood is
-    // still in L2 (sets whose records exceed L2).  First solve: all 19 coefficients of
+    // still in L2.  First solve: all 19 coefficients of
     // every field in place of its parked right-hand side, and the nine linear
     // and quadratic ones (which the correction is added to) in the slot's
     // column of the stash

@@ -441,10 +441,9 @@ struct FitArgs {
   // largest conditioning estimate exceeds refine_kappa, 1 every tile
   int32_t refine_mode;
   float refine_kappa;
-  // the corrected step of refined tiles in k_fit_refine over a queue (sets
-  // whose FP32 records fit in L2 and whose lambda varies) or inside the tile
-  // (larger sets: the tile's neighbourhood is still in L2 right after its
-  // main passes)
+  // the corrected step of refined tiles in k_fit_refine over a queue (small
+  // sets of varying lambda) or inside the tile, whose neighbourhood is still in
+  // L2 right after its main passes
   bool refine_queued;
   int32_t* rqueue;             // [n] fits queued for the corrected step
   int32_t* rq_len;             // their count (zeroed before the launch)
@@ -501,7 +500,6 @@ cudaError_t launch_fit_fp64(const FitArgs& a, FitMode mode, const int32_t* list,
                             const int32_t* list_len, const uint8_t* tmap, cudaStream_t st,
                             bool routed = false);
 int num_sms();
-size_t l2_bytes();  // L2 cache size of the current device (queried once)
 
 // Launch bookkeeping (measurement helpers, see include/phurbas_bench.h).
 void note_launch(int count = 1);

@@ -73,17 +73,6 @@ int num_sms() {
   return sms;
 }
 
-size_t l2_bytes() {
-  static int l2 = 0;
-  if (!l2) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess || l2 <= 0)
-      l2 = 64 << 20;
-  }
-  return static_cast<size_t>(l2);
-}
-
 phb_status launch_status(cudaError_t e) {
   if (e == cudaSuccess) e = cudaGetLastError();
   return e == cudaSuccess ? PHB_OK : PHB_ERR_CUDA;

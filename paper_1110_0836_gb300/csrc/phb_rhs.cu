@@ -91,7 +91,7 @@ cudaError_t gather_sorted(const phb_plan* p, const Grid& g, const double* pos, c
   return cudaGetLastError();
 }
 
-FitArgs fit_args(const phb_plan* plan, const phb_params* prm, void* ws, const int32_t* perm_out,
+FitArgs fit_args(const phb_plan* plan, const phb_params* prm, void* ws, int64_t fits, const int32_t* perm_out,
                  double* dudt, double* grad, double* hess, int32_t* fit_status,
                  int32_t* status_word) {
   FitArgs a;
@@ -124,11 +124,16 @@ FitArgs fit_args(const phb_plan* plan, const phb_params* prm, void* ws, const in
   a.status_word = status_word;
   a.refine_mode = prm->refine < 0 ? -1 : (prm->refine > 0 ? 1 : 0);
   a.refine_kappa = static_cast<float>(prm->refine_kappa > 0 ? prm->refine_kappa : 500.0);
-  // by size: the queue where the records fit in L2 and lambda varies (sets
-  // of one resolution, lattices above all, rarely refine: they skip the
-  // queue's launch and refine inside the tile when they do)
+  // by size: the queue for sets of fewer fits than kRefineQueued where lambda
+  // varies (sets of one resolution, lattices above all, rarely refine: they
+  // skip the queue's launch and refine inside the tile when they do).
+  // Right-hand sides in ms, queue / tile: tube 10,007 0.179 / 0.177, 40,000
+  // 0.207 / 0.218, 65,536 0.280 / 0.270, 200,000 0.677 / 0.684, 1M 3.25 / 3.24;
+  // shear layer 10,007 0.361 / 0.374, 40,000 0.440 / 0.446, 65,536 0.678 /
+  // 0.615, 200,000 1.38 / 1.34, 1M 4.9 / 4.6, 8M 32.8 / 28.5
+  constexpr int64_t kRefineQueued = 1 << 16;
   a.refine_queued = prm->refine_schedule == 1 ||
-                    (prm->refine_schedule != 2 && static_cast<size_t>(plan->n) * 96 <= l2_bytes() &&
+                    (prm->refine_schedule != 2 && fits < kRefineQueued &&
                      plan->lambda_max > 1.01 * plan->lambda_min);
   a.rqueue = region<int32_t>(plan, ws, R_RQUEUE);
   a.rq_len = a.queue_len + 6;
@@ -149,7 +154,8 @@ cudaError_t run_fit(const phb_plan* plan, const phb_params* prm, void* ws, FitMo
                     int32_t* fit_status, int32_t* status_word, cudaStream_t st,
                     const int32_t* list, const int32_t* list_len, int64_t list_cap,
                     const HostU* hu) {
-  FitArgs a = fit_args(plan, prm, ws, perm_out, dudt, grad, hess, fit_status, status_word);
+  FitArgs a = fit_args(plan, prm, ws, list ? list_cap : plan->n, perm_out, dudt, grad, hess, fit_status,
+                       status_word);
   if (hu && mode == FitMode::kRHS && !list && !perm_out && prm->precision != PHB_FP64) {
     a.u_host = hu->u_host;
     a.pc_y0 = hu->y0;
@@ -262,7 +268,7 @@ extern "C" int phb_fit_tc_experiment(const phb_plan* plan, const phb_params* prm
   const Grid g = make_grid(plan);
   cudaError_t e = gather_sorted(plan, g, pos, lambda, U, ws, status_word, st);
   if (e) return launch_status(e);
-  const FitArgs a = fit_args(plan, prm, ws, region<int32_t>(plan, ws, R_PERM), dudt, nullptr,
+  const FitArgs a = fit_args(plan, prm, ws, plan->n, region<int32_t>(plan, ws, R_PERM), dudt, nullptr,
                              nullptr, nullptr, status_word);
   e = launch_fit_tc(a, region<int2>(plan, ws, R_TPLAN), region<int32_t>(plan, ws, R_TSLOT),
                     region<uint16_t>(plan, ws, R_LSELF), region<uint8_t>(plan, ws, R_TMAP),
