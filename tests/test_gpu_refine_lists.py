@@ -36,3 +36,25 @@ def test_pairs_and_single_entries_agree(n, more):
         out.append(phb.mhd_rhs(plan, prm, pos, lam, Ut)[0].clone())
         assert plan.stats()["refined_tiles"] > 0
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("n,active", [(65_535, 0), (65_536, 0), (131_100, 65_535), (131_100, 65_536)])
+def test_either_side_of_the_queue(n, active):
+    """The default schedule on both sides of 65,536 fits, of a whole set and of an
+    active subset by listed slots, against both forced ones, bit for bit."""
+    phb = need_gpu()
+    w = workloads.shear_layer(n, seed=5)
+    n = w.n
+    pos, lam, Ut = phb.tensors_of(w)
+    plan = phb.Plan.for_workload(w)
+    phb.build_neighbors(plan, pos, lam)
+    idx = torch.tensor(np.random.default_rng(7).permutation(n)[:active].astype(np.int32), device="cuda")
+    out = []
+    for sched in ("auto", "queue", "tile"):
+        prm = phb.Params(gamma=w.gamma, refine="on", refine_schedule=sched)
+        if active:
+            out.append(phb.mhd_rhs_active(plan, prm, pos, lam, Ut, idx).clone())
+        else:
+            out.append(phb.mhd_rhs(plan, prm, pos, lam, Ut)[0].clone())
+        assert plan.stats()["refined_tiles"] > 0
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
