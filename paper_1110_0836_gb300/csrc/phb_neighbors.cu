@@ -888,10 +888,16 @@ __global__ void __launch_bounds__(T, 1152 / T) k_compact(const __grid_constant__
       for (int q = 0; q < m; ++q) ts_out[l0 + q] = t0 + q;
     }
     if (tid < cnt) {
+      // a slot that is in no cell (no finite position) or whose cell nothing
+      // marked has no staged record: index 0, which is one (its list is empty)
       const int s = s0 + tid;
-      const int j = marked_index(tarr, box_index(g, ts, cellc[s]));
-      const int o = s - cstart[j];  // (a slot without a finite position is in no cell)
-      lself[s] = static_cast<uint16_t>(base[j] + (static_cast<unsigned>(o) < static_cast<unsigned>(base[j + 1] - base[j]) ? o : 0));
+      const int k = box_index(g, ts, cellc[s]);
+      int self = 0;
+      if (bits[k >> 5] >> (k & 31) & 1u) {
+        const int j = marked_index(tarr, k), o = s - cstart[j];
+        if (static_cast<unsigned>(o) < static_cast<unsigned>(base[j + 1] - base[j])) self = base[j] + o;
+      }
+      lself[s] = static_cast<uint16_t>(self);
     }
   }
   // the tile's entries [e0, e1) as one flat range over the block (each
