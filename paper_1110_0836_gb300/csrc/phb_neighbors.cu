@@ -203,7 +203,7 @@ __device__ __forceinline__ Reach axis_reach_cells(const Grid& g, int a, int c, i
     q.wrap = false;
   } else {
     q.start = c - R;
-    q.count = 2 * R + 1;
+    q.count = max(2 * R + 1, 0);  // R = -1: no cells
     q.wrap = g.periodic[a] != 0;
   }
   return q;

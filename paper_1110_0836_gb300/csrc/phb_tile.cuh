@@ -41,9 +41,13 @@ struct TileArrays {
 };
 
 // Cells of reach of list radius r on axis a (covers every neighbour; see
-// the cell-size argument in the neighbour search).
+// the cell-size argument in the neighbour search); no more than the axis has.
+// A radius no reach belongs to (negative, infinite, 2^30 cells and more: a
+// lambda far outside the plan's range, which the build reports) gets -1, a
+// reach of no cells.
 __device__ __forceinline__ int reach_cells(const Grid& g, int a, double r) {
-  return static_cast<int>(ceil(r * g.inv_cell[a] * (1.0 + 1e-6)));
+  const int R = static_cast<int>(ceil(r * g.inv_cell[a] * (1.0 + 1e-6)));
+  return static_cast<unsigned>(R) < (1u << 30) ? min(R, g.ncell[a]) : -1;
 }
 
 // Box coordinate (0 .. dim-1) of global cell c on axis a.
