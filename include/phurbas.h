@@ -27,8 +27,9 @@
  *     re-ordered by cell, and results are returned in the caller's order.
  *   - The library allocates no device memory: all scratch lives in the
  *     caller-provided workspace `ws` of `ws_bytes` bytes, whose size is given
- *     by phb_workspace_size.  Neighbour lists live in the workspace between
- *     calls; a workspace belongs to one plan.
+ *     by phb_workspace_size.  It starts on a multiple of 16 bytes
+ *     (PHB_ERR_INVALID_ARG otherwise).  Neighbour lists live in the workspace
+ *     between calls; a workspace belongs to one plan.
  *   - Every call is asynchronous on `stream` (a cudaStream_t; NULL = legacy
  *     default stream) and performs no host synchronisation, so call sequences
  *     can be captured into CUDA graphs.

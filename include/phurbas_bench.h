@@ -46,7 +46,8 @@ int phb_trace_start(int32_t capacity);
  * written by every fit and step call (slot order, 24 floats per slot:
  * (xh, yh, zh, 0) (xl, yl, zl, 0) (rho, sigma, Vx, Vy)_h (..)_l
  * (Vz, Bx, By, Bz)_h (..)_l, with h = v rounded to FP32 and l = (v - h)
- * rounded to FP32), for tests that check them.  Host only.  Returns 0, or 1
+ * rounded to FP32), for tests that check them.  (In a workspace that does not
+ * start on a multiple of 32 bytes they lie 16 bytes further on.)  Host only.  Returns 0, or 1
  * for an invalid plan or NULL output. */
 int phb_record_region(const phb_plan* plan, size_t* offset, size_t* bytes);
 

@@ -30,7 +30,7 @@ enum Region {
   R_SPOS,        // double [3][n] positions, slot order
   R_SLAM,        // double [n]    lambda, slot order
   R_SU,          // double [8][n] fields, slot order
-  R_REC,         // float [n][24] FP32 hi/lo records
+  R_REC,         // float [n][24] FP32 hi/lo records (32-byte aligned)
   R_SCREEN,      // float4 [n]   wrapped FP32 positions for the neighbour screen
   R_NCNT,        // int32 [n+1]  neighbour counts
   R_OFF,         // int64 [n+1]  CSR offsets (slot order)
@@ -73,13 +73,19 @@ enum Region {
 };
 static_assert(R_COUNT <= 48, "ws_off has 48 entries");
 
+// A workspace starts on a multiple of 16 bytes; the records, read 32 bytes at a
+// time, start on the first multiple of 32 in their region.
+constexpr size_t kWsAlign = 16, kRecAlign = 32;
+
 template <typename T>
-__host__ __device__ inline T* region(const phb_plan* p, void* ws, Region r) {
-  return reinterpret_cast<T*>(static_cast<char*>(ws) + p->ws_off[r]);
+inline T* region(const phb_plan* p, void* ws, Region r) {
+  uintptr_t at = reinterpret_cast<uintptr_t>(ws) + p->ws_off[r];
+  if (r == R_REC) at = (at + kRecAlign - 1) & ~uintptr_t(kRecAlign - 1);
+  return reinterpret_cast<T*>(at);
 }
 template <typename T>
-__host__ __device__ inline const T* region(const phb_plan* p, const void* ws, Region r) {
-  return reinterpret_cast<const T*>(static_cast<const char*>(ws) + p->ws_off[r]);
+inline const T* region(const phb_plan* p, const void* ws, Region r) {
+  return region<T>(p, const_cast<void*>(ws), r);
 }
 
 // Plain-old-data view of the plan handed to kernels by value.

@@ -80,7 +80,7 @@ phb_status launch_status(cudaError_t e) {
 
 phb_status check_common(const phb_plan* plan, const void* ws, size_t ws_bytes, size_t need) {
   if (!plan || plan->n <= 0 || plan->ws_bytes == 0) return PHB_ERR_INVALID_ARG;
-  if (!ws) return PHB_ERR_INVALID_ARG;
+  if (!ws || reinterpret_cast<uintptr_t>(ws) % kWsAlign != 0) return PHB_ERR_INVALID_ARG;
   if (ws_bytes < need) return PHB_ERR_WORKSPACE;
   return PHB_OK;
 }
@@ -324,7 +324,7 @@ extern "C" phb_status phb_plan_init(phb_plan* p) {
   sz[R_SPOS] = 3 * n * 8;
   sz[R_SLAM] = n * 8;
   sz[R_SU] = 8 * n * 8;
-  sz[R_REC] = n * kRec * 4;
+  sz[R_REC] = n * kRec * 4 + kRecAlign - kWsAlign;
   sz[R_SCREEN] = n * 16;
   sz[R_NCNT] = (n + 1) * 4;
   sz[R_OFF] = (n + 1) * 8;
