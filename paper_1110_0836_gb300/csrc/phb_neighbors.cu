@@ -1153,6 +1153,10 @@ __global__ void __launch_bounds__(128, 10) k_adapt_scan(const __grid_constant__ 
   if (w >= n) return;
   const int s = static_cast<int>(w);
   const double lam = slam[s];
+  // for a lambda that is not a positive number every point's own comparisons
+  // decide (a NaN, an infinity and a zero have none to test)
+  const bool usual = finite64(lam) && __double2hiint(lam) >= 0x00100000;
+  const uint32_t each = usual ? rule.ask : 0xffffffffu;
   // FP32 radii with a margin: coordinates (screen_margin) and a few ulps of
   // r for offsets, squares and the radii themselves
   const float lamf = f32_of(lam);
@@ -1225,7 +1229,7 @@ __global__ void __launch_bounds__(128, 10) k_adapt_scan(const __grid_constant__ 
       const int kx = D.x[p], ky = D.y[p], kz = D.z[p];
       const uint32_t q = 1u << (kx * kx + ky * ky + kz * kz);
       ask = (rule.test & q) != 0u;
-      if (rule.ask & q) {
+      if (each & q) {
         const double rr = __dmul_rn(g.rf_factor, lam), hh = __dmul_rn(rr, 0.25);
         const double v = __dmul_rn(rule.vf, lam), in = __dsub_rn(rr, v);
         const double ox = __dmul_rn(static_cast<double>(kx), hh), oy = __dmul_rn(static_cast<double>(ky), hh),
