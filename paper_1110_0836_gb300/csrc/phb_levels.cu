@@ -21,7 +21,7 @@ __device__ __forceinline__ int level_of_step(double dt_max, double dt, int max_l
   const long long a = __double_as_longlong(dt_max), b = __double_as_longlong(dt);
   const int ea = static_cast<int>(a >> 52), eb = static_cast<int>(b >> 52);  // both > 0 or dt NaN
   int L = 0;
-  if (ea > 64 && eb > 64 && eb < 0x7ff) {
+  if (ea > 64 && ea < 0x7ff && eb > 64 && eb < 0x7ff) {
     constexpr long long kSig = (1ll << 52) - 1;
     L = ea - eb + ((a & kSig) > (b & kSig) ? 1 : 0);
     return L < 0 ? 0 : (L > max_level ? max_level : L);
