@@ -325,7 +325,9 @@ def gen():
     w("// In-place Cholesky of the packed normal matrix.  On return the packed")
     w("// array holds L (strict lower part; the diagonal entries keep M_kk) and")
     w("// inv_diag[k] = 1 / L_kk.  Returns the smallest pivot L_kk^2 seen (<= 0:")
-    w("// not positive definite).  MT / DT: arrays or array-like accessors.")
+    w("// not positive definite), or a NaN if the last one is (a NaN in M makes")
+    w("// one of its pivots and all later ones NaN).  MT / DT: arrays or array-like")
+    w("// accessors.")
     w("template <typename T, typename MT, typename DT>")
     w("__device__ __forceinline__ T mls_cholesky(MT& M, DT& inv_diag) {")
     w("  T minpiv = M[0];")
@@ -337,7 +339,7 @@ def gen():
             w(f"  {{ T s = M[{tri(j, j)}];")
             for k in range(j):
                 w(f"    s = fma(-M[{tri(j, k)}], M[{tri(j, k)}], s);")
-        w("    minpiv = s < minpiv ? s : minpiv;")
+        w("    minpiv = s >= minpiv ? minpiv : s;")
         w(f"    const T r = phb_rsqrt(s > T(0) ? s : T(1));")
         w(f"    inv_diag[{j}] = r;")
         for i in range(j + 1, NB):

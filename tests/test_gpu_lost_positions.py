@@ -3,8 +3,9 @@ their slots have no staged record of their own."""
 import numpy as np
 import pytest
 
+import oracle
 import workloads
-from _gpu import need_gpu, torch
+from _gpu import need_gpu, rhs_err, rhs_term_scales
 
 pytestmark = pytest.mark.gpu
 
@@ -43,3 +44,46 @@ def test_lost_slots_of_a_full_stage(spare):
     assert (st0 != 1).sum() > 80
     assert np.abs(g[..., keep] - g0).max() <= 1e-4 * np.abs(g0).max()
     assert (st[lost] == 1).all() and not g[..., lost].any()
+
+
+def lattice(seed):
+    """A lattice in storage order, and its lists' oracle."""
+    phb = need_gpu()
+    w = workloads.random_modes(12, seed=seed, amp=0.05)
+    plan = phb.Plan.for_workload(w)
+    pos, lam, U = phb.tensors_of(w)
+    phb.build_neighbors(plan, pos, lam)
+    phb.reorder(plan, pos, lam, U)
+    w.pos, w.lam, w.U = pos.cpu().numpy(), lam.cpu().numpy(), U.cpu().numpy()
+    phb.build_neighbors(plan, pos, lam)
+    return phb, w, plan, pos, lam, U
+
+
+def without(w, lost):
+    """Right-hand sides and their term scales from lists that leave `lost` out."""
+    box = oracle.box_of(w)
+    off, idx = oracle.neighbors(box, w.pos, w.lam)
+    keep = ~np.isin(idx, lost)
+    cut = np.concatenate([[0], np.cumsum(keep)])[off]
+    nb = (cut.astype(off.dtype), idx[keep])
+    exp, st = oracle.mhd_rhs(box, w.pos, w.lam, w.U, nb, gamma=w.gamma)
+    g, h, _ = oracle.mls_derivs(box, w.pos, w.lam, w.U, nb, gamma=w.gamma)
+    assert not st.any()
+    return exp, rhs_term_scales(w.U, g, h, w.gamma)
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("value", [np.nan, -np.nan, np.inf])
+@pytest.mark.parametrize("slot", ["first"])
+def test_position_lost_after_the_build(axis, value, slot):
+    """A neighbour whose position is not a number or infinite when the fit
+    runs is left out of every fit that lists it, in both precisions."""
+    phb, w, plan, pos, lam, U = lattice(82)
+    lost = 128 * 3 + {"first": 0}[slot]
+    exp, sc = without(w, [lost])
+    other = np.setdiff1d(np.arange(w.n), [lost])
+    pos[axis, lost] = value
+    for prec, tol in (("fp64", 1e-12), ("fp32_mixed", 1e-5)):
+        out, _ = phb.mhd_rhs(plan, phb.Params(gamma=w.gamma, precision=prec), pos, lam, U)
+        e = rhs_err(out.cpu().numpy()[:, other], exp[:, other], sc)
+        assert e.max() < tol, (prec, e)
