@@ -40,8 +40,12 @@
 namespace phb {
 namespace {
 
+struct Near32 {
+  float lo[3], far[3];  // box corner; 2^20 box lengths
+};
 struct Per32 {
   float len_h[3], len_l[3], inv_len[3], len[3];
+  Near32 near;
 };
 
 __device__ __forceinline__ float hl(float ah, float al, float bh, float bl) {
@@ -558,17 +562,37 @@ __device__ __forceinline__ void first_slots(const FitArgs& a, const int32_t* slo
   for (int u = 0; u < kStageBatch; ++u) first[u] = tid + u * T < a.g.stage_cap ? slots[tid + u * T] : -1;
 }
 
+// Whether the records of a tile may be staged relative to slot s: its fields
+// finite, its position within 2^20 box lengths of the box (the differences'
+// rounding grows with it: a lost particle's would be NaNs, one at 1e30 would
+// leave nothing of its neighbours').
+__device__ __forceinline__ bool may_refer(const float4* rec, const Near32& b, int s) {
+  const float4 x = rec[6 * s], f = rec[6 * s + 2], g = rec[6 * s + 4];
+  const float u = fmaf(0.f, f.x + f.y, fmaf(0.f, f.z + f.w, 0.f * (g.x + g.y) + 0.f * (g.z + g.w)));  // 0 or a NaN
+  return fabsf(x.x - b.lo[0]) < b.far[0] && fabsf(x.y - b.lo[1]) < b.far[1] &&
+         fabsf(x.z - b.lo[2]) < b.far[2] && u == 0.f;
+}
+
+// The first such slot of a tile, or its middle one where there is none.
+__device__ __noinline__ int other_reference(const float4* rec, Near32 b, int s0, int cnt) {
+  for (int k = 0; k < cnt; ++k)
+    if (may_refer(rec, b, s0 + k)) return s0 + k;
+  return s0 + (cnt >> 1);
+}
+
 // Stage a tile's neighbourhood (count records, slots from the plan) in shared
-// memory: offsets and field differences relative to the tile's middle slot
-// sr, from the FP32 hi/lo records.  All T threads call it; no barrier inside.
+// memory: offsets and field differences relative to slot sr, the middle one of
+// its cnt slots from s0 (or one that may serve), from the FP32 hi/lo records.  All T threads call it; no barrier inside.
 // Returns whether this thread staged an offset of a quarter box length or
 // more on a periodic axis (the tile's differences then need the wrap).
 template <int T>
 __device__ __forceinline__ bool stage_tile(const FitArgs& a, const Per32& P, const int32_t* slots,
-                                           const int (&first)[kStageBatch], int sr, int count,
-                                           float4* stage, int tid) {
+                                           const int (&first)[kStageBatch], int s0, int cnt,
+                                           int count, float4* stage, int tid) {
   bool far = false;
   const float4* rec = reinterpret_cast<const float4*>(a.rec);
+  int sr = s0 + (cnt >> 1);
+  if (!may_refer(rec, P.near, sr)) sr = other_reference(rec, P.near, s0, cnt);
   // records relative to the tile's middle particle: the staged FP32 offsets
   // and field differences round to at most half the tile's extent
   const float4 rh = rec[6 * sr], rl = rec[6 * sr + 1];
@@ -687,7 +711,7 @@ __device__ __forceinline__ void fit_tile(const FitArgs& a, const Per32& P, const
   // the neighbourhood planned by the neighbour build: one gather per staged record
   const bool fb = tp.y != 0;
   if (!fb) {
-    const bool far = stage_tile<T>(a, P, slots, staged_first, s0 + (cnt_tile >> 1), tp.x, stage, tid);
+    const bool far = stage_tile<T>(a, P, slots, staged_first, s0, cnt_tile, tp.x, stage, tid);
     const bool wfar = __any_sync(0xffffffffu, far);
     if ((tid & 31) == 0) sh.wfar[tid >> 5] = wfar ? 1 : 0;
   } else if (tid == 0 && !listed) {
@@ -1057,7 +1081,7 @@ __global__ void __launch_bounds__(T, 2) k_gram_tc(const FitArgs a, const Per32 P
     const int32_t* slots = ta.tslot + static_cast<int64_t>(tile) * a.g.stage_cap;
     int first[kStageBatch];
     first_slots<T>(a, slots, tid, first);
-    stage_tile<T>(a, P, slots, first, s0 + (cnt_tile >> 1), tp.x, stage, tid);
+    stage_tile<T>(a, P, slots, first, s0, cnt_tile, tp.x, stage, tid);
   }
   __syncthreads();
   const bool unweighted = a.weight_kind == 1;
@@ -1228,6 +1252,8 @@ Per32 make_per32(const Grid& g) {
     P.len_l[a] = g.periodic[a] ? static_cast<float>(g.len[a] - static_cast<double>(h)) : 0.f;
     P.inv_len[a] = g.periodic[a] ? static_cast<float>(1.0 / g.len[a]) : 0.f;
     P.len[a] = h;
+    P.near.lo[a] = static_cast<float>(g.lo[a]);
+    P.near.far[a] = h * 1048576.f;
   }
   return P;
 }

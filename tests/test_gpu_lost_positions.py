@@ -5,7 +5,7 @@ import pytest
 
 import oracle
 import workloads
-from _gpu import need_gpu, rhs_err, rhs_term_scales
+from _gpu import need_gpu, rhs_err, rhs_term_scales, sets_of, torch
 
 pytestmark = pytest.mark.gpu
 
@@ -74,16 +74,61 @@ def without(w, lost):
 
 @pytest.mark.parametrize("axis", [0, 1, 2])
 @pytest.mark.parametrize("value", [np.nan, -np.nan, np.inf])
-@pytest.mark.parametrize("slot", ["first"])
+@pytest.mark.parametrize("slot", ["first", "middle"])
 def test_position_lost_after_the_build(axis, value, slot):
     """A neighbour whose position is not a number or infinite when the fit
     runs is left out of every fit that lists it, in both precisions."""
     phb, w, plan, pos, lam, U = lattice(82)
-    lost = 128 * 3 + {"first": 0}[slot]
+    lost = 128 * 3 + {"first": 0, "middle": 64}[slot]   # a tile is staged relative to its middle slot
     exp, sc = without(w, [lost])
     other = np.setdiff1d(np.arange(w.n), [lost])
     pos[axis, lost] = value
     for prec, tol in (("fp64", 1e-12), ("fp32_mixed", 1e-5)):
         out, _ = phb.mhd_rhs(plan, phb.Params(gamma=w.gamma, precision=prec), pos, lam, U)
         e = rhs_err(out.cpu().numpy()[:, other], exp[:, other], sc)
+        assert e.max() < tol, (prec, e)
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("field", [0, 3, 7])
+def test_field_lost(field, value):
+    """A field that is not finite, of a tile's middle particle, reaches the
+    particles that list it and no others."""
+    phb, w, plan, pos, lam, U = lattice(83)
+    lost = 128 * 5 + 64
+    exp, sc = without(w, [])
+    got = sets_of(*phb.export_neighbors(plan))
+    far = np.array([i for i in range(w.n) if i != lost and lost not in got[i]])
+    assert 32 < w.n - far.size < 80
+    U[field, lost] = value
+    for prec, tol in (("fp64", 1e-12), ("fp32_mixed", 1e-5)):
+        out, _ = phb.mhd_rhs(plan, phb.Params(gamma=w.gamma, precision=prec), pos, lam, U)
+        e = rhs_err(out.cpu().numpy()[:, far], exp[:, far], sc)
+        assert e.max() < tol, (prec, e)
+
+
+@pytest.mark.parametrize("side", [12, 26])
+def test_positions_far_away_before_the_build(side):
+    """Finite positions beyond 2^53 cells are counted to an edge cell, whose tile
+    they must not spoil: fits of the particles that do not list one are those of
+    the set without them, in both precisions.  (Sets of both searches.)"""
+    phb = need_gpu()
+    w = workloads.random_modes(side, seed=84, amp=0.05)
+    rng = np.random.default_rng(9)
+    # the caller's first particles lie about the cells that far positions are counted to
+    lost = np.concatenate([np.arange(0, 60, 2), rng.permutation(w.n)[:30]])
+    exp, sc = without(w, lost)
+    pos, lam, U = (torch.tensor(x, device="cuda") for x in (w.pos, w.lam, w.U))
+    at = torch.tensor(lost, device="cuda")
+    pos[:, at] = torch.tensor(rng.choice([1e30, -3e200, 1e300, 2.2e25, -7.7e18], (3, lost.size)), device="cuda")
+    plan = phb.Plan.for_workload(w)
+    phb.build_neighbors(plan, pos, lam, check_capacity=False)
+    got = sets_of(*phb.export_neighbors(plan))
+    is_lost = np.zeros(w.n, bool)
+    is_lost[lost] = True
+    far = np.array([i for i in range(w.n) if not is_lost[i] and not is_lost[got[i]].any()])
+    assert far.size > w.n // 2
+    for prec, tol in (("fp64", 1e-12), ("fp32_mixed", 1e-5)):
+        out, _ = phb.mhd_rhs(plan, phb.Params(gamma=w.gamma, precision=prec), pos, lam, U)
+        e = rhs_err(out.cpu().numpy()[:, far], exp[:, far], sc)
         assert e.max() < tol, (prec, e)
