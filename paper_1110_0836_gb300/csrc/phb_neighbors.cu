@@ -70,10 +70,16 @@ __global__ void k_scatter(int n, const int32_t* __restrict__ keys, const int32_t
 // Thread per particle: its rank among the particles of its cell is the number
 // of them with a smaller caller index (the cells' members come from the
 // atomic scatter in arbitrary order).  That is quadratic in a cell's members
-// (~12), so a cell of more than kBigCell - a clump, or the key of the particles
-// without a finite position - is listed in one sweep of the
-// block that holds its first scattered member.
-constexpr int kBigCell = 2048;
+// (~12), so a crowded one - a clump, or the key of the particles without a
+// finite position - is listed in one sweep over all n keys by the block that
+// holds its first scattered member.  The sweep takes n x 2 ns (200,000
+// particles 0.23 ms, 1M 1.05, 8M 16.2), the ranks 35 ns per member and up to 10 ps
+// per pair of them (builds in ms, ranks / sweep: 8M with 8,000 members 7.8 / 23.4,
+// 32,000: 15.0 / 23.4, 64,000: 30.1 / 23.4, 256,000: 200 / 23.2; 1M with 8,000: 1.38
+// / 1.99, 16,000: 2.20 / 1.99; 200,000 with 4,000: 0.39 / 0.53, 8,000: 0.55 / 0.52).
+__device__ __forceinline__ bool crowded(int members, int n) {
+  return static_cast<int64_t>(members) * members > 256 * static_cast<int64_t>(n);
+}
 
 __global__ void __launch_bounds__(kThreads) k_rank_cells(int n, int32_t nkeys, const int32_t* __restrict__ keys,
                                                          const int32_t* __restrict__ cell_start,
@@ -85,7 +91,7 @@ __global__ void __launch_bounds__(kThreads) k_rank_cells(int n, int32_t nkeys, c
   if (i < n) {
     k = keys[i];
     const int a = cell_start[k], b = k < nkeys ? cell_start[k + 1] : n;
-    if (b - a <= kBigCell) {
+    if (!crowded(b - a, n)) {
       int rank = 0;
       for (int t = a; t < b; ++t) rank += scattered[t] < i ? 1 : 0;
       perm[a + rank] = i;
