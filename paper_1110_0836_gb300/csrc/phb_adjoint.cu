@@ -37,6 +37,8 @@
 // factor, its diagonal's reciprocals and the fitted coefficients once
 // (kRecord) and the adjoint then starts from that record (kStored) instead of
 // re-accumulating the moments and right-hand sides.
+#include <algorithm>
+
 #include "phb_fit64.cuh"
 #include "phb_mhd.cuh"
 
@@ -100,11 +102,16 @@ __device__ __forceinline__ int first_slot(const int64_t* off, int n, int64_t e0)
   return lo;
 }
 
-// Slots [first, last) of the chunk: those whose lists start in its span of the
-// entries (a list is shorter than n, so their entries fit span + n rows).
+// Slots [first, last) of the chunk: those whose lists start in its part of the
+// entries, which as few chunks as hold them share evenly (a list is shorter
+// than n, so a chunk's entries fit span + n rows; the later chunks of a capacity
+// that the lists do not need are empty).
 __device__ __forceinline__ void chunk_slots(const AdjArgs& a, int& first, int& last) {
-  first = a.chunk == 0 ? 0 : first_slot(a.off, a.n, a.chunk * a.span);
-  last = a.chunk == a.chunks - 1 ? a.n : first_slot(a.off, a.n, (a.chunk + 1) * a.span);
+  const int64_t total = a.off[a.n] < a.g.capacity ? a.off[a.n] : a.g.capacity;
+  const int64_t used = total > a.span ? (total + a.span - 1) / a.span : 1;
+  const int64_t part = (total + used - 1) / used;
+  first = a.chunk == 0 ? 0 : (a.chunk < used ? first_slot(a.off, a.n, a.chunk * part) : a.n);
+  last = a.chunk + 1 < used ? first_slot(a.off, a.n, (a.chunk + 1) * part) : a.n;
 }
 
 // Adjoint of the right-hand side at one particle.  In: point values u, the
@@ -541,11 +548,12 @@ __global__ void __launch_bounds__(128) k_adj_gather(const __grid_constant__ AdjA
       add_rows(sorted[wid], m - base < 32 ? m - base : 32);
     }
   }
+  const bool done = a.chunk == a.chunks - 1;
+  if (m == 0 && !done) return;  // (of an empty chunk, all)
   const double s1 = __shfl_down_sync(0xffffffffu, acc, kTerms);
   const double s2 = __shfl_down_sync(0xffffffffu, acc, 2 * kTerms);
   acc += s1 + s2;
   // columns 0..6: Ubar of fields 1..7, 7..9: xbar; Ubar of field 0 has own terms only
-  const bool done = a.chunk == a.chunks - 1;
   const int k = lane < kTerms ? lane + 1 : 0;
   if (lane > kTerms) return;
   double* sum = a.acc + k * N + t;
@@ -606,7 +614,9 @@ phb_status adjoint_impl(int mode, const phb_plan* plan, const phb_params* prm, c
   a.status_word = status_word;
   a.span = adjoint_rows(plan) - n;
   a.chunk = 0;
-  a.chunks = static_cast<int32_t>(plan->nbr_capacity > a.span ? (plan->nbr_capacity + a.span - 1) / a.span : 1);
+  // (no more entries than the capacity, and than every particle naming every other)
+  const int64_t most = std::min<int64_t>(plan->nbr_capacity, int64_t(n) * (n - 1));
+  a.chunks = static_cast<int32_t>(std::max<int64_t>((most + a.span - 1) / a.span, 1));
   const size_t smem = size_t(kSlots) * kT * sizeof(double);
   const unsigned grid = static_cast<unsigned>(num_sms());
   const auto kernel = mode == kRecompute ? k_adjoint<kRecompute>

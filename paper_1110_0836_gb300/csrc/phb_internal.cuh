@@ -111,11 +111,13 @@ Grid make_grid(const phb_plan* p);
 // bricks, else 0.
 int64_t brick_words(const phb_plan* p);
 
-// Rows (list entries) of the adjoint's term buffer: all list entries of sets up
-// to 2^17 particles (2^23 rows at most), else 28 per particle - the entries
-// then go through it in chunks of rows - n (a list is shorter than n), two at
-// ~52 neighbours, in no more memory than a record of seeds and coefficients
-// per particle took.
+// Rows (list entries) of the adjoint's term buffer: 28 per particle, 2.4 KB, less
+// than a stored record's 2.7 - the entries go through it in chunks of rows - n (a
+// list is shorter than n), two at ~52 neighbours.  Small sets get up to 2^20
+// rows (88 MB): a chunk takes 1.9 ms however few its particles, and 2^20 entries
+// are those of one pass of the adjoint's grid, 19,456 particles (gradient of
+// 4,096 particles 2.0 ms in one chunk, 4.0 in two; of 97,336, with 28 rows, 12.0
+// ms against 11.7 in one chunk of all entries, which took 370 MB more).
 int64_t adjoint_rows(const phb_plan* p);
 
 __device__ __forceinline__ float phb_rsqrt(float x) { return rsqrtf(x); }

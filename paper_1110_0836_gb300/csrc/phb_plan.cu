@@ -58,8 +58,8 @@ int64_t brick_words(const phb_plan* p) {
 }
 
 int64_t adjoint_rows(const phb_plan* p) {
-  const int64_t all = std::max<int64_t>(p->nbr_capacity, 1) + p->n, some = 28 * p->n;
-  return p->n > int64_t(1) << 17 ? some : std::max(some, std::min<int64_t>(all, int64_t(1) << 23));
+  const int64_t all = std::max<int64_t>(p->nbr_capacity, 1) + p->n;
+  return std::max(28 * p->n, std::min<int64_t>(all, int64_t(1) << 20));
 }
 
 int num_sms() {
