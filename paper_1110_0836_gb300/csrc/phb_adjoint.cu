@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kT, 1) k_adjoint(const __grid_constant__ AdjAr
       mls_assemble(m, M);
       singular = cnt < kNB;
       if (!singular) {
-        float mkk[kNB];
+        double mkk[kNB];
         chol_panel<0, 4>(my, mkk, singular);
         chol_panel<4, 4>(my, mkk, singular);
         chol_panel<8, 5>(my, mkk, singular);

@@ -62,10 +62,10 @@ struct Num {
 // stride 32), the columns before them done: the panel in registers, so that
 // its independent FMAs cover the shared-memory loads (loops of dot products
 // through shared memory took 290 cycles per FMA, this form ~90).  The diagonal
-// slots take 1 / L_kk, mkk the diagonal of M in FP32.  A Jacobi-scaled pivot
+// slots take 1 / L_kk, mkk the diagonal of M.  A Jacobi-scaled pivot
 // below 1e-12 (cond(M) above ~1e12) is treated as singular.
 template <int C0, int W>
-__device__ __forceinline__ void chol_panel(double* my, float (&mkk)[kNB], bool& singular) {
+__device__ __forceinline__ void chol_panel(double* my, double (&mkk)[kNB], bool& singular) {
   constexpr int R = kNB - C0;
   double v[W][R];
   double d[W];
@@ -74,7 +74,7 @@ __device__ __forceinline__ void chol_panel(double* my, float (&mkk)[kNB], bool& 
 #pragma unroll
     for (int r = c; r < R; ++r) v[c][r] = my[(tri0(C0 + r) + C0 + c) * 32];
     d[c] = v[c][c];
-    mkk[C0 + c] = f32_of(d[c]);
+    mkk[C0 + c] = d[c];
   }
 #pragma unroll 1
   for (int k = 0; k < C0; ++k) {

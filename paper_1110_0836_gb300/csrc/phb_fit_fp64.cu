@@ -9,10 +9,10 @@
 // integer work and FP32 work disappear behind them.  A lattice fit (52
 // neighbours) is 267 FP64 instructions per neighbour (80 moments, 7 x 19
 // right-hand sides, 54 for offsets, weight and monomials) and ~3,900 for the
-// factorisation and the solves: 18,500, or 8.3-9.5 ms for 262,144 particles.
-// Comparisons, the test for a periodic wrap and the conditioning estimate run
-// on the integer and FP32 pipes for that reason.  Measured: 11.5 ms (FP64 pipe
-// 66% busy); with all sums in shared memory and two warps per SM it was 23.0 ms
+// factorisation and the solves, ~700 for the estimate: 19,200, or 8.6-9.9 ms for 262,144 particles.
+// Comparisons and the test for a periodic wrap run on the integer pipe for that
+// reason.  Measured: 11.8 ms (before the conditioning estimate was FP64 11.5, FP64
+// pipe 66% busy); with all sums in shared memory and two warps per SM it was 23.0 ms
 // (35%).
 //
 // Two ways to fit a particle, bit-identical (each sum and each substitution
@@ -51,30 +51,33 @@ constexpr int kWI = kWM + kNM;           // 1 / L_kk
 constexpr int kWarpSlots = kWI + kNB;
 static_assert(kWarpSlots <= kSlots * 32, "the warp form runs in the thread form's shared memory");
 
+// sqrt(M_kk) of a positive pivot's diagonal entry.
+__device__ __forceinline__ double root64(double m) { return __dmul_rn(m, rsqrt(m)); }
+
 // Estimate of ||M_s^-1||_inf of the Jacobi-scaled matrix (as mls_inv_norm_est,
-// the back substitution by columns) in FP32 from the factor in a thread's
-// column and the diagonal mkk of M: it only picks the fits that take the
-// corrected step, and costs 700 FP64 instructions otherwise.  The factor is
-// read twice (volatile) rather than kept: 190 registers.
-__device__ __forceinline__ float inv_norm_est(const double* my, const float (&mkk)[kNB]) {
+// the back substitution by columns) from the factor in a thread's column and the
+// diagonal mkk of M; it picks the fits that take the corrected step.  (Formed in
+// FP32 it saved 0.27 of 12.28 ms for 262,144 particles, but the entries of a
+// tight cluster's M underflow there.)  The factor is read twice (volatile) rather
+// than kept: 190 registers.
+__device__ __forceinline__ double inv_norm_est(const double* my, const double (&mkk)[kNB]) {
   const volatile double* L = my;
-  float y[kNB], inv[kNB];
+  double y[kNB];
 #pragma unroll
   for (int i = 0; i < kNB; ++i) {
-    float t = 0.f;
+    double t = 0.0;
 #pragma unroll
-    for (int k = 0; k < i; ++k) t = fmaf(f32_of(L[(tri0(i) + k) * 32]), y[k], t);
-    const float sq = sqrtf(mkk[i]);
-    inv[i] = f32_of(L[(tri0(i) + i) * 32]);
-    y[i] = ((t > 0.f ? -sq : sq) - t) * inv[i];
+    for (int k = 0; k < i; ++k) t = fma(L[(tri0(i) + k) * 32], y[k], t);
+    const double sq = root64(mkk[i]);
+    y[i] = ((t > 0.0 ? -sq : sq) - t) * L[(tri0(i) + i) * 32];
   }
-  float mx = 0.f;
+  double mx = 0.0;
 #pragma unroll
   for (int k = kNB - 1; k >= 0; --k) {
-    y[k] *= inv[k];
-    mx = fmaxf(mx, fabsf(y[k]) * sqrtf(mkk[k]));
+    y[k] *= L[(tri0(k) + k) * 32];
+    mx = fmax(mx, fabs(y[k]) * root64(mkk[k]));
 #pragma unroll
-    for (int i = 0; i < k; ++i) y[i] = fmaf(-f32_of(L[(tri0(k) + i) * 32]), y[k], y[i]);
+    for (int i = 0; i < k; ++i) y[i] = fma(-L[(tri0(k) + i) * 32], y[k], y[i]);
   }
   return mx;
 }
@@ -112,7 +115,7 @@ __device__ __noinline__ void write_rhs(const FitArgs& a, int s, int dst, const M
 // the fit needs the corrected step.
 template <FitMode MODE>
 __device__ __forceinline__ bool fit_thread(const FitArgs& a, const Box64& bx, int slot, bool routed,
-                                           float refine_above, double* my) {
+                                           double refine_above, double* my) {
   constexpr int f0 = MODE == FitMode::kRHS ? 1 : 0;  // the RHS never needs the density fit
   const int64_t n = a.n;
   const int s = slot < 0 ? 0 : slot;
@@ -136,7 +139,7 @@ __device__ __forceinline__ bool fit_thread(const FitArgs& a, const Box64& bx, in
   mls_assemble(m, M);
   bool singular = cnt < kNB;
   if (!singular) {
-    float mkk[kNB];
+    double mkk[kNB];
     chol_panel<0, 4>(my, mkk, singular);
     chol_panel<4, 4>(my, mkk, singular);
     chol_panel<8, 5>(my, mkk, singular);
@@ -285,26 +288,28 @@ __device__ __forceinline__ int warp_sums(const FitArgs& a, const Box64& bx, cons
 }
 
 // inv_norm_est with a row per lane (each sum in its order).
-__device__ __forceinline__ float warp_inv_norm_est(const double* W, int lane) {
+__device__ __forceinline__ double warp_inv_norm_est(const double* W, int lane) {
   const double* L = W + kWL;
   const int i = lane < kNB ? lane : kNB - 1;
-  const float inv = f32_of(W[kWI + i]);
-  const float sq = sqrtf(f32_of(W[kWM + mls_moment_index(i, i)]));
-  float s = 0.f, y = 0.f;
+  const double inv = W[kWI + i];
+  const double sq = root64(W[kWM + mls_moment_index(i, i)]);
+  double s = 0.0, y = 0.0;
 #pragma unroll
   for (int k = 0; k < kNB; ++k) {
-    if (lane == k) y = ((s > 0.f ? -sq : sq) - s) * inv;
-    const float yk = __shfl_sync(0xffffffffu, y, k);
-    if (i > k) s = fmaf(f32_of(L[tri0(i) + k]), yk, s);
+    if (lane == k) y = ((s > 0.0 ? -sq : sq) - s) * inv;
+    const double yk = __shfl_sync(0xffffffffu, y, k);
+    if (i > k) s = fma(L[tri0(i) + k], yk, s);
   }
 #pragma unroll
   for (int k = kNB - 1; k >= 0; --k) {
     if (lane == k) y *= inv;
-    const float xk = __shfl_sync(0xffffffffu, y, k);
-    if (i < k) y = fmaf(-f32_of(L[tri0(k) + i]), xk, y);
+    const double xk = __shfl_sync(0xffffffffu, y, k);
+    if (i < k) y = fma(-L[tri0(k) + i], xk, y);
   }
-  const float x = lane < kNB ? fabsf(y) * sq : 0.f;
-  return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));
+  double mx = lane < kNB ? fabs(y) * sq : 0.0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  return mx;
 }
 
 // Substitutions of all fields at once, four lanes per field (rows i = q mod 4);
@@ -340,7 +345,7 @@ __device__ __forceinline__ void warp_solve(const double* W, const double* rhs, i
 // One particle by one warp (all lanes call it with the same s).
 template <FitMode MODE>
 __device__ __forceinline__ void fit_warp(const FitArgs& a, const Box64& bx, const WarpTab& tab, int s,
-                                         bool routed, float refine_above, double* W) {
+                                         bool routed, double refine_above, double* W) {
   constexpr int f0 = MODE == FitMode::kRHS ? 1 : 0;
   const int lane = threadIdx.x & 31;
   const double lam = a.slam[s];
@@ -387,7 +392,7 @@ __device__ __forceinline__ void fit_warp(const FitArgs& a, const Box64& bx, cons
   }
   bool refine = false;
   if (!singular) {
-    const float est = warp_inv_norm_est(W, lane);
+    const double est = warp_inv_norm_est(W, lane);
     refine = kNB * est > refine_above;
     __syncwarp();
     double v[5];
@@ -467,7 +472,7 @@ __global__ void __launch_bounds__(kT, 1) k_fit_fp64(const __grid_constant__ FitA
   double* W = sm + wid * kSlots * 32;
   // fits routed from the FP32-mixed path need ~1e-5: FP64 normal equations
   // meet that up to cond(M) ~ 1e9; the FP64 path itself targets ~1e-12
-  const float refine_above = routed ? 1e9f : 1e4f;
+  const double refine_above = routed ? 1e9 : 1e4;
   auto slot = [&](int w) {
     if (list) return w < total ? list[w] : -1;
     if (w >= total) return -1;
