@@ -445,10 +445,10 @@ phb_status phb_rhs_adjoint(const phb_plan* plan, const phb_params* params, const
 /* Stored-factorisation variant of phb_rhs_adjoint (not in the paper; offered
  * to compare memory and time against recomputation).
  * phb_adjoint_record_bytes(plan): bytes of the per-particle record, 343
- * doubles per particle = the Jacobi-scaled Cholesky factor of the 19 x 19
- * normal matrix (190), its scaling (19), the fitted coefficients of the seven
- * fields V, B, sigma (7 x 19) and a singular flag, [343][n] in the
- * workspace's slot order.  0 for an invalid plan.
+ * doubles per particle = the Cholesky factor L of the 19 x 19 normal matrix
+ * with 1 / L_kk on its diagonal (190), 19 words that are not used, the fitted
+ * coefficients of the seven fields V, B, sigma (7 x 19) and a singular flag,
+ * [343][n] in the workspace's slot order.  0 for an invalid plan.
  * phb_adjoint_record: FP64 fits of every particle with the lists of the last
  * build; writes the record (device, caller-owned, >= record_bytes).
  * phb_rhs_adjoint_stored: the same result as phb_rhs_adjoint, starting from

@@ -174,23 +174,11 @@ def gen():
     w("constexpr int kQuad0 = 10;  // first quadratic index (xx, xy, xz, yy, yz, zz)")
     w("")
     # monomials
-    w("// q^gamma for the 19 basis monomials, and w q^beta for beta in {0} U basis.")
-    w("template <typename T>")
-    w("__device__ __forceinline__ void mls_monomials(T x, T y, T z, T wt, T (&qg)[kNB], T (&wq)[kNB + 1]) {")
-    w("  const T xx = x * x, xy = x * y, xz = x * z, yy = y * y, yz = y * z, zz = z * z;")
     vals = {(1, 0, 0): "x", (0, 1, 0): "y", (0, 0, 1): "z", (2, 0, 0): "xx", (1, 1, 0): "xy",
             (1, 0, 1): "xz", (0, 2, 0): "yy", (0, 1, 1): "yz", (0, 0, 2): "zz"}
     cubic_expr = {(3, 0, 0): "xx * x", (2, 1, 0): "xx * y", (2, 0, 1): "xx * z", (1, 2, 0): "xy * y",
                   (1, 1, 1): "xy * z", (1, 0, 2): "xz * z", (0, 3, 0): "yy * y", (0, 2, 1): "yy * z",
                   (0, 1, 2): "yz * z", (0, 0, 3): "zz * z"}
-    for i, e in enumerate(BASIS):
-        expr = cubic_expr.get(e, vals.get(e))
-        w(f"  qg[{i}] = {expr};  // {name(e)}")
-    w("  wq[0] = wt;")
-    for i in range(NB):
-        w(f"  wq[{i + 1}] = wt * qg[{i}];")
-    w("}")
-    w("")
     w("// q^gamma for the 19 basis monomials, w, and w q^beta for the ten cubic")
     w("// betas only (all that mls_accum_moments reads); wq[11..19] are not set.")
     w("template <typename T>")
@@ -250,20 +238,6 @@ def gen():
     for a, alpha in enumerate(MOMENTS):
         b, g = split(alpha)
         w(f"  m[{a}] = fma(wq[{b + 1}], qg[{g}], m[{a}]);  // {name(alpha)}")
-    w("}")
-    w("")
-    w("// b[beta] += w q^beta du for the 19 basis monomials.")
-    w("template <typename T>")
-    w("__device__ __forceinline__ void mls_accum_rhs(const T (&wq)[kNB + 1], T du, T (&b)[kNB]) {")
-    for i in range(NB):
-        w(f"  b[{i}] = fma(wq[{i + 1}], du, b[{i}]);")
-    w("}")
-    w("")
-    w("// b[beta] += q^beta (w du) for the 19 basis monomials (weight folded into du).")
-    w("template <typename T>")
-    w("__device__ __forceinline__ void mls_accum_rhs_basis(const T (&qg)[kNB], T wdu, T (&b)[kNB]) {")
-    for i in range(NB):
-        w(f"  b[{i}] = fma(qg[{i}], wdu, b[{i}]);")
     w("}")
     w("")
     w("// Normal matrix, packed lower triangle: M[tri(r,c)] = m[e_r + e_c].")

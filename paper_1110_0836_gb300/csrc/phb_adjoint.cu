@@ -23,19 +23,18 @@
 // part of the entries: the particles are taken in chunks of consecutive slots.
 //
 // What bounds it: the FP64 pipe (see phb_fit_fp64.cu).  Per neighbour the fit
-// takes 267 FP64 instructions and the backward pass ~500 (2 x 7 x 19 products
-// with the seeds, 180 for the degree-6 polynomial and its gradient by nested
-// multiplication); forming every entry's terms once and passing them through
+// takes 267 FP64 instructions and the backward pass ~500 (266 products with the
+// seeds, 162 FMAs and 40 others for the degree-6 polynomial and its gradient by
+// nested multiplication, the rest offsets and weights); forming every entry's terms once and passing them through
 // memory (80 B written and read per entry, 0.3 ms per 262,144 particles) costs
 // less than forming them a second time for the neighbour.  Four warps per SM
 // (213 doubles of shared memory per thread).  Measured, 262,144 particles:
-// gradient 62.4 -> 30.0 ms (before: each entry's terms formed again in the gather, 84
+// gradient 62.3 -> 28.2 ms (before: each entry's terms formed again in the gather, 84
 // tabulated monomials, seeds in global memory).
 //
 // By default the factorisation is recomputed here (nothing is stored by the
 // forward call); the stored variant records, per particle, the Cholesky
-// factor, its diagonal's reciprocals and the fitted coefficients once
-// (kRecord) and the adjoint then starts from that record (kStored) instead of
+// factor and the fitted coefficients once (kRecord) and the adjoint then starts from that record (kStored) instead of
 // re-accumulating the moments and right-hand sides.
 #include <algorithm>
 
@@ -54,9 +53,9 @@ constexpr int kSlotMbar = kNFit * kNB;
 constexpr int kSlots = kSlotMbar + kNM;
 static_assert(kSlots >= kNT && size_t(kSlots) * kT * 8 <= 227 * 1024, "shared memory of a block");
 // record of one particle's forward fit, [k][n] layout: factor (190, 1 / L_kk on
-// its diagonal), 1 / L_kk (19), coefficients c_f (7 x 19), then 1 = singular /
-// 0 = regular
-constexpr int kRecFac = 0, kRecInvd = kNT, kRecCoef = kNT + kNB, kRecFlag = kRecCoef + kNFit * kNB;
+// its diagonal), 19 words not used (they keep the record's size), coefficients
+// c_f (7 x 19), then 1 = singular / 0 = regular
+constexpr int kRecFac = 0, kRecCoef = kNT + kNB, kRecFlag = kRecCoef + kNFit * kNB;
 constexpr int kRecWords = kRecFlag + 1;
 constexpr int kTerms = 10;  // an entry's row: dUbar of fields 1..7, dbar
 enum AdjMode { kRecompute = 0, kRecord = 1, kStored = 2 };
@@ -282,7 +281,6 @@ __global__ void __launch_bounds__(kT, 1) k_adjoint(const __grid_constant__ AdjAr
         if (!singular) {
 #pragma unroll 10
           for (int k = 0; k < kNT; ++k) a.rec[(kRecFac + k) * N + s] = my[k * 32];
-          for (int k = 0; k < kNB; ++k) a.rec[(kRecInvd + k) * N + s] = my[(tri0(k) + k) * 32];
 #pragma unroll 10
           for (int k = 0; k < kNFit * kNB; ++k) a.rec[(kRecCoef + k) * N + s] = c[k];
         }
