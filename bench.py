@@ -51,16 +51,11 @@ KERNEL_FLOP_PER_NEIGHBOUR = 2 * (80 + 7 * 19)
 KERNEL_FLOP_PER_PARTICLE = 2 * (1140 + 7 * 171 + 7 * 36) + 100
 # DRAM bytes (read + write) per launch of the fused fit from one-kernel ncu
 # captures of the kernel as it is built now (profiles/fit_mixed_traffic.md):
-# workload name -> (bytes per launch, how).  Workloads too large to capture
-# under the size rule are captured on a smaller set of the same recipe and
-# scaled by the particles processed.  Absent = null.
+# workload name -> (bytes per launch, how).  Absent = null.
 FIT_TRAFFIC = {
     "random_modes_64^3": (68728064 + 2951168, "ncu, this workload, one launch"),
     "shock_tube_1048576": (492819456 + 300109312, "ncu, this workload, one launch"),
-    "shear_layer_8000000": (8 * (481017344 + 285916928),
-                            "ncu on the 1,000,000-particle set of the same recipe with the "
-                            "corrected step in the tiles (the 8M set's schedule), x 8 "
-                            "(particles processed)"),
+    "shear_layer_8000000": (3900000000 + 2500000000, "ncu, this workload, one launch"),
 }
 
 
@@ -515,8 +510,8 @@ def run_ours(args):
     step_ms_max = aggregate_max(step_ms, world, dev)
     value = world * 2 * n / (step_ms_max * 1e-3)
 
-    # the fit is two kernels: the fused fit and the corrected step of the fits
-    # of refined tiles (an empty queue on a lattice)
+    # the fit is one kernel, or two where the corrected step of the refined
+    # tiles' fits runs over a queue
     mixed_avg = float(np.mean(fit_ms)) if fit_ms else float("nan")
     refine_avg = float(np.sum(refine_ms)) / len(fit_ms) if (refine_ms and fit_ms) else 0.0
     fit_avg = mixed_avg + refine_avg
@@ -533,9 +528,9 @@ def run_ours(args):
                 "frac": achieved / peak, "traffic": None if tr is None else tr[0],
                 "traffic_unit": "DRAM bytes read + written per launch (ncu, profiles/)",
                 "traffic_how": None if tr is None else tr[1],
-                "kernel": f"{kname}<kRHS, {int(plan.c.tile)}> + k_fit_refine<kRHS, {int(plan.c.tile)}> "
-                          "(fused FP32 MLS fit + MHD RHS, then the corrected step of the fits of "
-                          "refined tiles)",
+                "kernel": f"{kname}<kRHS, {int(plan.c.tile)}> (fused FP32 MLS fit + MHD RHS"
+                          + (f") + k_fit_refine<kRHS, {int(plan.c.tile)}> (the corrected step of the fits "
+                             "of refined tiles)" if refine_ms else ", the corrected step of refined tiles in it)"),
                 "launch_ms": fit_avg, "launches": len(fit_ms),
                 "launch_ms_parts": {kname: mixed_avg, "k_fit_refine": refine_avg},
                 "timed_on": "eager pass over the timed steps (CUDA events on the launching stream)"

@@ -11,9 +11,8 @@
 // right-hand sides, 54 for offsets, weight and monomials) and ~3,900 for the
 // factorisation and the solves, ~700 for the estimate: 19,200, or 8.6-9.9 ms for 262,144 particles.
 // Comparisons and the test for a periodic wrap run on the integer pipe for that
-// reason.  Measured: 11.8 ms (before the conditioning estimate was FP64 11.5, FP64
-// pipe 66% busy); with all sums in shared memory and two warps per SM it was 23.0 ms
-// (35%).
+// reason.  Measured: 12.0 ms (FP64 pipe 67% busy); with all sums in shared memory
+// and two warps per SM it was 23.0 ms (35%).
 //
 // Two ways to fit a particle, bit-identical (each sum and each substitution
 // takes its terms in the same order):

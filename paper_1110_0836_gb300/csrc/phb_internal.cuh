@@ -134,7 +134,7 @@ __device__ __forceinline__ bool finite64(double x) {
   return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
 }
 
-// v truncated to FP32 on the integer pipe.
+// v truncated to FP32 on the integer pipe (NaNs and infinities: the largest float).
 __device__ __forceinline__ float f32_of(double v) {
   const unsigned hi = static_cast<unsigned>(__double2hiint(v));
   const unsigned mag = hi & 0x7fffffffu;

@@ -130,7 +130,8 @@ FitArgs fit_args(const phb_plan* plan, const phb_params* prm, void* ws, int64_t 
   // Right-hand sides in ms, queue / tile: tube 10,007 0.179 / 0.177, 40,000
   // 0.207 / 0.218, 65,536 0.280 / 0.270, 200,000 0.677 / 0.684, 1M 3.25 / 3.24;
   // shear layer 10,007 0.361 / 0.374, 40,000 0.440 / 0.446, 65,536 0.678 /
-  // 0.615, 200,000 1.38 / 1.34, 1M 4.9 / 4.6, 8M 32.8 / 28.5
+  // 0.615, 200,000 1.38 / 1.34, 1M 4.9 / 4.6, 8M 32.8 / 28.5.  (Up to 200,000 the two
+  // lie within 5%, either way, but for the layer at 65,536; beyond the tiles win.)
   constexpr int64_t kRefineQueued = 1 << 16;
   a.refine_queued = prm->refine_schedule == 1 ||
                     (prm->refine_schedule != 2 && fits < kRefineQueued &&
